@@ -161,9 +161,10 @@ typedef struct henry_config {
                            rounding floor). Default 1e-14 */
   int res_rows;         /* rows of cells one thread of the residual/Jacobian
                            kernel walks (its tile height per row group),
-                           1..64; 0 (default): 8. A schedule knob for the
-                           autotuner: it trades blocks per sample against
-                           recomputed faces at tile edges */
+                           1..64; 0 (default): 2..16 by the size of the
+                           grid. A schedule knob for the autotuner: it
+                           trades warps per sample against recomputed faces
+                           at tile edges */
   int discretisation;   /* HENRY_DISC_CELL (default) or HENRY_DISC_VERTEX:
                            the vertex-centred variant of section 2.3 (box
                            method with partial upwinding; see
@@ -395,20 +396,9 @@ int henry_residual_jacobian(const henry_config* cfg, int nx, int ny, double tau,
  * it), and latency-critical loops where an allocation could synchronise the
  * device or fail part-way. Arguments, layouts, outputs and errors are those
  * of henry_residual_jacobian; the caller still provides every input and
- * output buffer.
- * Scratch: 5 doubles per cell and sample in a file-scope device array of
- * 2^20 doubles (8 MiB), held by every GPU that loads the library until the
- * process exits; B * nx * ny above 209715 cells is rejected with
- * HENRY_E_INVALID (as is B > HENRY_MAX_BATCH). The first call on a device
- * looks up the array's device address (cudaGetSymbolAddress) with that
- * device current and caches it for the process; make that first call
- * before any stream capture. The cached address does not survive
- * cudaDeviceReset() (the module is reloaded at a new address): do not call
- * this entry point on a device after resetting it. Every call shares the array and it keeps
- * the last call's contents; each call writes every scratch element it reads
- * before reading it, so nothing needs to start at zero. Calls that overlap
- * on the GPU (on different streams, or from different host threads) race on
- * the array and must be serialised by the caller. */
+ * output buffer. The evaluation is one kernel without scratch memory; B *
+ * nx * ny above 209715 cells is rejected with HENRY_E_INVALID (as is B >
+ * HENRY_MAX_BATCH). */
 int henry_residual_jacobian_noalloc(const henry_config* cfg, int nx, int ny, double tau, int B,
                                     const double* phi, const double* K, const double* qin,
                                     const double* p, const double* c, const double* c_old,

@@ -23,7 +23,7 @@ cudaError_t launch_field_stats(unsigned long long* ctr, int nx, int ny, int B, c
 cudaError_t launch_residual_jacobian(const Phys& P, const Geom& G, double tau, int B,
                                      const double* phi, const double* K, const double* qin,
                                      const double* p, const double* c, const double* c_old,
-                                     double* R, double* J, double* scratch, cudaStream_t s);
+                                     double* R, double* J, cudaStream_t s);
 int or_status(const int* src, int* dst, int B, unsigned long long* ctr, cudaStream_t s);
 constexpr int kProbeThreads = 152 * 8 * 256;
 cudaError_t probe_fp64(int reps, double* out, cudaStream_t s, double* tflops);
@@ -634,14 +634,8 @@ int henry_residual_jacobian(const henry_config* cfg, int nx, int ny, double tau,
   henry::Phys P{cfg->rho0, cfg->rho1 - cfg->rho0, cfg->mu, cfg->g, cfg->D, cfg->K0, cfg->phi0,
                 cfg->q0, cfg->Lx, cfg->Ly};
   henry::Geom G{nx, ny, cfg->Lx / nx, cfg->Ly / ny};
-  cudaStream_t s = (cudaStream_t)stream;
-  double* scratch = nullptr;
-  CKR(cudaMallocAsync((void**)&scratch, sizeof(double) * 5 * (size_t)B * nx * ny, s));
-  cudaError_t e = henry::launch_residual_jacobian(P, G, tau, B, phi, K, qin, p, c, c_old, R, J,
-                                                  scratch, s);
-  cudaError_t e2 = cudaFreeAsync(scratch, s);
-  CKR(e);
-  CKR(e2);
+  CKR(henry::launch_residual_jacobian(P, G, tau, B, phi, K, qin, p, c, c_old, R, J,
+                                      (cudaStream_t)stream));
   return HENRY_OK;
 }
 

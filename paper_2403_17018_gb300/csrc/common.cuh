@@ -134,25 +134,60 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   return s;
 }
 
-// Tiling of the face-based residual kernel (see k_resjac).
+// Tiling of k_residual (residual.cuh): lpr lanes share a row of a warp (C columns each), gpw row groups
+// per warp, R rows per group; ntx x nty warps cover a sample.
 struct ResTile {
-  int TX, GR, R;    // columns per tile, row groups per block, rows per thread
-  int ntx, nty;     // tiles per sample in x and y
+  int lpr, gpw, R, ntx, nty;
+  __host__ __device__ int warps() const { return ntx * nty; }
 };
 
-// rmax: most rows a thread walks (more rows per thread: fewer blocks, fewer
-// tile-edge recomputations of the south face; fewer: more parallelism for
-// small batches). 0 selects the default, 8.
-__host__ inline ResTile make_res_tile(int nx, int ny, int rmax = 0) {
+// rows 0 selects the tile height from the grid alone (never from the batch:
+// the partial sums that decide convergence keep their order whatever the
+// batch is). A tile evaluates its south faces again, so tall tiles do less
+// work; short ones give a small batch more warps. Measured (us), residual
+// only: 32x16 cells x 1 sample 12 with 2 rows of 2 columns, 18 (2 rows) and 29
+// (4 rows) of 4 columns; x 1024 samples 57, 61, 49; 128x64 x 64 61 with 2 rows,
+// 47 with 4, 57 with 8; 512x256 x 16 194 with 8, 166 with 16; 1024x512 x 16 661
+// with 8, 717 with 16. With the Jacobian (FP32): 32x16 x 1 16 with 2 rows, 27
+// with 4; 128x64 x 64 94 with 2, 89 with 4, 80 with 8, but x 16 25, 29, 47;
+// 1024x512 x 16 978 with 8, 967 with 16.
+__host__ inline ResTile make_res_tile(int nx, int ny, int C, int rows, bool jac) {
   ResTile t;
-  if (rmax <= 0) rmax = 8;
-  t.TX = nx < kBlock ? nx : kBlock;
-  t.GR = kBlock / t.TX;
-  int rows = (ny + t.GR - 1) / t.GR;        // rows per thread if one tile covered all
-  t.R = rows < rmax ? rows : rmax;
-  t.ntx = (nx + t.TX - 1) / t.TX;
-  t.nty = (ny + t.GR * t.R - 1) / (t.GR * t.R);
+  const int lanes = (nx + C - 1) / C;
+  t.lpr = lanes < 32 ? lanes : 32;
+  t.gpw = 32 / t.lpr;
+  t.ntx = (lanes + 31) / 32;
+  const int64_t ncell = (int64_t)nx * ny;
+  if (rows <= 0)
+    rows = jac ? (ncell <= 4096 ? 2 : (ncell <= 65536 ? 4 : (ncell <= 262144 ? 8 : 16)))
+               : (ncell <= 4096 ? 2 : (ncell <= 65536 ? 4 : (ncell <= 262144 ? 16 : 8)));
+  const int most = (ny + t.gpw - 1) / t.gpw;
+  t.R = rows < most ? rows : most;
+  t.nty = (ny + t.gpw * t.R - 1) / (t.gpw * t.R);
   return t;
 }
+
+// Inputs of k_residual.
+struct ResArgs {
+  const double* p;        // [B][ncell] reduced pressure (full pressure with OWN)
+  const double* c;
+  const double* c_old;    // old time level (otherwise)
+  const double* phi;
+  const double* K;        // OWN only
+  const double* tx;       // face constants (without OWN), dx and dy halved; the
+  const double* dx;       //   last column's east slots hold the right side's
+  const double* ty;
+  const double* dy;
+  const float4* tf;       // (tx, dx, ty, dy), not halved (FP32 Jacobian)
+  const double* qin;      // [B][ny]
+  const double* vt;       // V phi / tau (without OWN); (V phi / tau) rho_old and
+  const double* mo;       //   (V phi / tau) rho_old c_old (solver's residual)
+  const double* so;
+  const int* active;      // [B] or null
+  const int* refresh;     // [B] or null: samples to skip
+  double* partial;        // [B][warps] sums of R_p^2 + R_c^2, or null
+  double* qx;             // face fluxes (WANT_J of the multigrid layout), or null
+  double* qy;
+};
 
 }  // namespace henry

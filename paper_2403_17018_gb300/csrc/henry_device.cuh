@@ -8,9 +8,8 @@
 //   F_m   = A q rho_up                                          (Eq. 1 flux)
 //   F_s   = A [ q (rho c)_up - rho_bar phi_f D (c_U - c_L)/d ]  (Eq. 2 flux, Eq. 5)
 // K_f, phi_f harmonic means, rho_bar arithmetic mean of rho(c) (Eq. 4),
-// upwind from L when q >= 0, else from U. Both cells evaluate a face with the
-// same canonical orientation and the same operations, so the two residual
-// contributions cancel exactly in floating point.
+// upwind from L when q >= 0, else from U. A face's flux is evaluated once, in
+// the canonical orientation, and enters its two cells with opposite signs.
 // Boundaries: left x=0 prescribed mass inflow rho0 q_in(y), no advected salt,
 // diffusive Dirichlet c=0 at hx/2; right x=Lx Dirichlet p = rho1 g (Ly - y)
 // at hx/2, advected values upwinded with c=1 on inflow, diffusive Dirichlet
@@ -368,7 +367,7 @@ __device__ __forceinline__ double inflow_at(const Phys& P, int model, int n_xi, 
 // Face constants of cell (i, j): east face (if any) and north face (if any).
 // The last column's east slots hold the right side's coefficients, 2 A K_P
 // / (mu hx) and 2 A phi_P D / hx (the Dirichlet side at hx/2), for kernels
-// that treat the right side as one more face (k_resid); the others compute
+// that treat the right side as one more face (k_residual); the others compute
 // them from K and phi and read tx, dx only where an east neighbour exists.
 __device__ __forceinline__ void face_constants(const Phys& P, const Geom& G, int i, int j,
                                                const double* __restrict__ phi,

@@ -53,12 +53,18 @@ __device__ __forceinline__ void store_operator(T* __restrict__ Jb, int ncell, co
 #pragma unroll
   for (int q = 1; q <= 4; ++q) {
     const T a = Jc[4 * q], b = Jc[4 * q + 1], c = Jc[4 * q + 2], e = Jc[4 * q + 3];
-    Jb[(int64_t)(4 * q + 0) * ncell] = d[0] * a + d[1] * c;
-    Jb[(int64_t)(4 * q + 1) * ncell] = d[0] * b + d[1] * e;
-    Jb[(int64_t)(4 * q + 2) * ncell] = d[2] * a + d[3] * c;
-    Jb[(int64_t)(4 * q + 3) * ncell] = d[2] * b + d[3] * e;
+    Jb[(int64_t)(4 * q + 0) * ncell] = fma(d[0], a, d[1] * c);
+    Jb[(int64_t)(4 * q + 1) * ncell] = fma(d[0], b, d[1] * e);
+    Jb[(int64_t)(4 * q + 2) * ncell] = fma(d[2], a, d[3] * c);
+    Jb[(int64_t)(4 * q + 3) * ncell] = fma(d[2], b, d[3] * e);
   }
 }
+
+}  // namespace henry
+
+#include "residual.cuh"
+
+namespace henry {
 
 // ---------------------------------------------------------------------------
 // set-up kernels (once per solve)
@@ -109,10 +115,13 @@ static __global__ void k_coarsen_fields(unsigned long long* ctr, Geom Gf, Geom G
   Kc[idx] = 0.25 * (Kf[f0] + Kf[f0 + 1] + Kf[f0 + Gf.nx] + Kf[f0 + Gf.nx + 1]);
 }
 
+// dxh, dyh (optional): the halves of dx, dy; tf (optional): all four in FP32.
 static __global__ void k_face_consts(unsigned long long* ctr, Phys P, Geom G, int B,
                               const double* __restrict__ phi, const double* __restrict__ K,
                               double* __restrict__ tx, double* __restrict__ dx,
-                              double* __restrict__ ty, double* __restrict__ dy) {
+                              double* __restrict__ ty, double* __restrict__ dy,
+                              double* __restrict__ dxh, double* __restrict__ dyh,
+                              float4* __restrict__ tf) {
   HENRY_COUNT_LAUNCH(ctr);
   const int64_t n = (int64_t)B * G.ncell();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -121,7 +130,17 @@ static __global__ void k_face_consts(unsigned long long* ctr, Phys P, Geom G, in
   const int cell = (int)(idx - (int64_t)b * G.ncell());
   const int j = cell / G.nx, i = cell - j * G.nx;
   const int64_t o = (int64_t)b * G.ncell();
-  face_constants(P, G, i, j, phi + o, K + o, tx[idx], dx[idx], ty[idx], dy[idx]);
+  double a, d, e, f;
+  face_constants(P, G, i, j, phi + o, K + o, a, d, e, f);
+  tx[idx] = a;
+  dx[idx] = d;
+  ty[idx] = e;
+  dy[idx] = f;
+  if (dxh) {
+    dxh[idx] = 0.5 * d;
+    dyh[idx] = 0.5 * f;
+  }
+  if (tf) tf[idx] = make_float4((float)a, (float)d, (float)e, (float)f);
 }
 
 // Initial state c = 0; the Newton guess for p is seawater hydrostatics,
@@ -147,7 +166,7 @@ static __global__ void k_init_state(unsigned long long* ctr, Phys P, Geom G, int
 // per time step
 // ---------------------------------------------------------------------------
 // Start of an implicit Euler step: c_old = c^{n-1} (with mo / so given, also
-// the old-time storage terms of k_resid). With `extrapolate`, from
+// the old-time storage terms of k_residual). With `extrapolate`, from
 // the third step on (both u^{n-1} and u^{n-2} are solutions; the first
 // step's pressure guess is not) the Newton initial guess is extrapolated
 // linearly in time, u = 2 u^{n-1} - u^{n-2}, with c clamped to [0, 1]
@@ -216,7 +235,7 @@ static __global__ void k_begin_step(unsigned long long* ctr, Geom G, int B, doub
   p_prev[idx] = pn;
   if (mo) {
     // storage of the old time level, fixed for the whole step: (V phi / tau)
-    // rho(c_old) and (V phi / tau) rho(c_old) c_old (k_resid)
+    // rho(c_old) and (V phi / tau) rho(c_old) c_old (k_residual)
     const double vt = vtau * phi[idx];
     const double m = vt * (rho0 + drho * cn);
     mo[idx] = m;
@@ -245,368 +264,7 @@ static __global__ void k_end_step(unsigned long long* ctr, int* __restrict__ ste
   if (threadIdx.x == 0) *step += 1;
 }
 
-// FP64 residual of the finest grid and its Jacobian in the multigrid type T,
-// face by face. Tiling: a block covers TX columns x (GR * R) rows of one
-// sample; thread t takes column t % TX and walks R rows of row group t / TX.
-// Per cell the thread evaluates its east and north faces only: the west
-// face comes from the left neighbour thread through shared memory (or is
-// evaluated again at a tile edge) and the south face is the north face of
-// the previous row, kept in registers (evaluated once per column at the
-// bottom of a row group). Each face is evaluated with the canonical
-// orientation, so both cells see bitwise the same flux.
-// MG layout (NATURAL = false): writes b = -R, x = 0, J (colour-split), the
-// face fluxes qx (east / right side) and qy (north), one partial sum of
-// R_p^2 + R_c^2 per block. NATURAL = true: writes R [B][2][ncell] and J
-// [B][20][ncell] in natural cell order (FP64), for tests. WANT_J = false:
-// the residual outputs only (defect-correction iterations that reuse the
-// operators). refresh (optional, per sample): samples with refresh[b] == 0
-// are skipped.
-template <typename T, bool NATURAL, bool WANT_J = true>
-__global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 2 : 3)
-k_resjac(unsigned long long* ctr, Phys P, Geom G, double vtau, int B, ResTile tl,
-         const double* __restrict__ p, const double* __restrict__ c,
-         const double* __restrict__ c_old, const double* __restrict__ phi,
-         const double* __restrict__ K, const double* __restrict__ tx,
-         const double* __restrict__ dx, const double* __restrict__ ty,
-         const double* __restrict__ dy, const double* __restrict__ qin,
-         const int* __restrict__ active, T* __restrict__ J, T* __restrict__ bvec,
-         T* __restrict__ xvec, double* __restrict__ partial, double* __restrict__ qx,
-         double* __restrict__ qy, const int* __restrict__ refresh) {
-  HENRY_COUNT_LAUNCH(ctr);
-  __shared__ double shF[2][kBlock];
-  __shared__ T shD[8][kBlock];   // face derivatives (unused, and removed, when !WANT_J)
-  __shared__ double shr[kBlock / 32];
-  const int b = blockIdx.y;
-  if (!NATURAL && (!active[b] || (refresh && !refresh[b]))) return;
-  const int nx = G.nx, ny = G.ny, ncell = G.ncell(), half = G.half();
-  const int t = threadIdx.x;
-  const int col = t % tl.TX, rg = t / tl.TX;
-  const int bx = blockIdx.x % tl.ntx, by = blockIdx.x / tl.ntx;
-  const int i = bx * tl.TX + col;
-  const int j0 = by * tl.GR * tl.R + rg * tl.R;
-  const bool thr = rg < tl.GR && i < nx;
-  const int64_t o = (int64_t)b * ncell;
-  const double* pb_ = p + o;
-  const double* cb_ = c + o;
-  const double gdy = P.g * G.hy;
-  const double A = G.hy;
-  const double dcoL = 2.0 * A * P.D / G.hx;      // times phi_P
-  const double tRf = 2.0 * A / (P.mu * G.hx);    // times K_P
-  double v = 0.0;
-  // south face of the first row (halo), as L = S, U = P
-  double FmS = 0.0, FsS = 0.0;
-  FaceD<T> dS;
-  double pP = 0.0, cP = 0.0;
-  if (thr && j0 < ny) {
-    pP = pb_[j0 * nx + i];
-    cP = cb_[j0 * nx + i];
-    if (j0 > 0) {
-      const int id = (j0 - 1) * nx + i;
-      double q;
-      face_flux<T, WANT_J, false, true>(P, pb_[id], cb_[id], pP, cP, ty[o + id], dy[o + id], gdy, q,
-                                        FmS, FsS, dS);
-    }
-  }
-  for (int r = 0; r < tl.R; ++r) {
-    const int j = j0 + r;
-    const bool cv = thr && j < ny;
-    const int id = j * nx + i;
-    double FmE = 0.0, FsE = 0.0, qE = 0.0;
-    FaceD<T> dE;
-    T dR[4];   // right side derivatives (dF/du_P)
-    double phiP = 0.0, pN = 0.0, cN = 0.0;
-    if (cv) {
-      phiP = phi[o + id];
-      if (i < nx - 1) {
-        face_flux<T, WANT_J, false, false>(P, pP, cP, pb_[id + 1], cb_[id + 1], tx[o + id],
-                                           dx[o + id], 0.0, qE, FmE, FsE, dE);
-      } else {
-        const double pbd = P.drho * P.g * (P.Ly - (j + 0.5) * G.hy);
-        right_face<T, WANT_J, false>(P, pP, cP, tRf * K[o + id], dcoL * phiP, pbd, qE, FmE, FsE, dR);
-      }
-      shF[0][t] = FmE;
-      shF[1][t] = FsE;
-      if (WANT_J) {
-        shD[0][t] = dE.mLp; shD[1][t] = dE.mLc; shD[2][t] = dE.mUp; shD[3][t] = dE.mUc;
-        shD[4][t] = dE.sLp; shD[5][t] = dE.sLc; shD[6][t] = dE.sUp; shD[7][t] = dE.sUc;
-      }
-    }
-    __syncthreads();
-    if (cv) {
-      // west face (L = W, U = P)
-      double FmW = 0.0, FsW = 0.0;
-      FaceD<T> dW;
-      if (i > 0) {
-        if (col > 0) {
-          FmW = shF[0][t - 1];
-          FsW = shF[1][t - 1];
-          if (WANT_J) {
-            dW.mLp = shD[0][t - 1]; dW.mLc = shD[1][t - 1]; dW.mUp = shD[2][t - 1]; dW.mUc = shD[3][t - 1];
-            dW.sLp = shD[4][t - 1]; dW.sLc = shD[5][t - 1]; dW.sUp = shD[6][t - 1]; dW.sUc = shD[7][t - 1];
-          }
-        } else {
-          double q;
-          face_flux<T, WANT_J, false, false>(P, pb_[id - 1], cb_[id - 1], pP, cP, tx[o + id - 1],
-                                             dx[o + id - 1], 0.0, q, FmW, FsW, dW);
-        }
-      }
-      // north face (L = P, U = N)
-      double FmN = 0.0, FsN = 0.0, qN = 0.0;
-      FaceD<T> dN;
-      if (j < ny - 1) {
-        pN = pb_[id + nx];
-        cN = cb_[id + nx];
-        face_flux<T, WANT_J, false, true>(P, pP, cP, pN, cN, ty[o + id], dy[o + id], gdy, qN, FmN,
-                                          FsN, dN);
-      }
-      // accumulation
-      const double vt = vtau * phiP;
-      const double rho = P.rho0 + P.drho * cP;
-      const double cO = c_old[o + id];
-      const double rho_o = P.rho0 + P.drho * cO;
-      double Rp = vt * (rho - rho_o) + FmE + FmN - FmW - FmS;
-      double Rc = vt * (rho * cP - rho_o * cO) + FsE + FsN - FsW - FsS;
-      T Jc[20];
-#pragma unroll
-      for (int m = 0; m < 20; ++m) Jc[m] = (T)0;
-      Jc[1] = (T)(vt * P.drho);
-      Jc[3] = (T)(vt * (rho + P.drho * cP));
-      if (i > 0) {
-        Jc[0] -= dW.mUp; Jc[1] -= dW.mUc; Jc[2] -= dW.sUp; Jc[3] -= dW.sUc;
-        Jc[4] = -dW.mLp; Jc[5] = -dW.mLc; Jc[6] = -dW.sLp; Jc[7] = -dW.sLc;
-      } else {
-        // left side: fixed freshwater inflow, diffusion to c = 0 at hx/2
-        const double dco = dcoL * phiP;
-        const double rb = 0.5 * (rho + P.rho0);
-        Rp += -A * P.rho0 * qin[(int64_t)b * ny + j];
-        Rc += dco * rb * cP;
-        if (WANT_J) Jc[3] += (T)(dco * (0.5 * P.drho * cP + rb));
-      }
-      if (i < nx - 1) {
-        Jc[0] += dE.mLp; Jc[1] += dE.mLc; Jc[2] += dE.sLp; Jc[3] += dE.sLc;
-        Jc[8] = dE.mUp; Jc[9] = dE.mUc; Jc[10] = dE.sUp; Jc[11] = dE.sUc;
-      } else {
-        Jc[0] += dR[0]; Jc[1] += dR[1]; Jc[2] += dR[2]; Jc[3] += dR[3];
-      }
-      if (j > 0) {
-        Jc[0] -= dS.mUp; Jc[1] -= dS.mUc; Jc[2] -= dS.sUp; Jc[3] -= dS.sUc;
-        Jc[12] = -dS.mLp; Jc[13] = -dS.mLc; Jc[14] = -dS.sLp; Jc[15] = -dS.sLc;
-      }
-      if (j < ny - 1) {
-        Jc[0] += dN.mLp; Jc[1] += dN.mLc; Jc[2] += dN.sLp; Jc[3] += dN.sLc;
-        Jc[16] = dN.mUp; Jc[17] = dN.mUc; Jc[18] = dN.sUp; Jc[19] = dN.sUc;
-      }
-      if (NATURAL) {
-        double* Rn = (double*)bvec + (int64_t)b * 2 * ncell;
-        Rn[id] = Rp;
-        Rn[ncell + id] = Rc;
-        if (WANT_J && J) {
-          T* Jn = J + (int64_t)b * 20 * ncell + id;
-#pragma unroll
-          for (int m = 0; m < 20; ++m) Jn[(int64_t)m * ncell] = Jc[m];
-        }
-      } else {
-        const int cs = cs_pos(i, j, nx, half);
-        const int64_t ob = (int64_t)b * 2 * ncell;
-        T* Jb = J + (int64_t)b * kJP * ncell + cs;
-        T d[4];   // Dinv of the operator the multigrid will use
-        if (WANT_J) {
-          store_operator<T>(Jb, ncell, Jc, d);
-        } else {
-#pragma unroll
-          for (int m = 0; m < 4; ++m) d[m] = Jb[(int64_t)m * ncell];
-        }
-        const T mp = (T)(-Rp), mc = (T)(-Rc);
-        bvec[ob + cs] = d[0] * mp + d[1] * mc;
-        bvec[ob + ncell + cs] = d[2] * mp + d[3] * mc;
-        xvec[ob + cs] = (T)0;
-        xvec[ob + ncell + cs] = (T)0;
-        qx[o + id] = qE;
-        qy[o + id] = qN;
-      }
-      v += Rp * Rp + Rc * Rc;
-      // the north face is the next row's south face
-      FmS = FmN;
-      FsS = FsN;
-      dS = dN;
-      pP = pN;
-      cP = cN;
-    }
-    __syncthreads();
-  }
-  if (!NATURAL) {
-    const double s = block_sum(v, shr);
-    if (threadIdx.x == 0) partial[(int64_t)b * gridDim.x + blockIdx.x] = s;
-  }
-}
-
-// FP64 residual of the finest grid alone, for the defect-correction
-// iterations that keep their operators (operator reuse): the same discrete
-// residual as k_resjac, arranged for GB300's narrow FP64 pipe, where every
-// FP64 warp instruction costs the same pipe time whether one lane or 32
-// are active (so the kernel avoids divergent FP64 work):
-//  * per-cell constants: vt = V phi / tau and the old-time storage terms
-//    mo = vt rho(c_old), so = mo c_old from k_begin_step, so the storage part
-//    is a = vt rho, R_p = a - mo, R_c = a c - so;
-//  * rho and rho c of a cell are formed once: the east neighbour's come from
-//    the next lane (shuffle), the north neighbour's become the next row's;
-//  * the west face is the east face of the previous lane; across a warp
-//    edge both the neighbour's state and the face travel through shared
-//    memory (two block barriers per row); only tile edges recompute;
-//  * the right side is one more face, to the Dirichlet values (p_b, c = 1),
-//    with the coefficients face_constants keeps in the last column;
-//  * a face's mean density and its gravity term share c_L + c_U.
-// Writes b = -Dinv R with the stored Dinv, x = 0, the face fluxes qx, qy
-// and one partial sum of R_p^2 + R_c^2 per block; same tiling as k_resjac.
-template <typename T>
-__global__ void __launch_bounds__(kBlock)
-k_resid(unsigned long long* ctr, Phys P, Geom G, int B, ResTile tl,
-        const double* __restrict__ p, const double* __restrict__ c,
-        const double* __restrict__ vt, const double* __restrict__ mo,
-        const double* __restrict__ so, const double* __restrict__ phi,
-        const double* __restrict__ tx, const double* __restrict__ dx,
-        const double* __restrict__ ty, const double* __restrict__ dy,
-        const double* __restrict__ qin, const int* __restrict__ active, const T* __restrict__ J,
-        T* __restrict__ bvec, T* __restrict__ xvec, double* __restrict__ partial,
-        double* __restrict__ qx, double* __restrict__ qy) {
-  HENRY_COUNT_LAUNCH(ctr);
-  constexpr int kW = kBlock / 32;
-  __shared__ double shS[4][kW];    // lane 0's p, c, rho, rho c for the previous warp's lane 31
-  __shared__ double shF[2][kW];    // lane 31's east-face fluxes for the next warp's lane 0
-  __shared__ double shr[kW];
-  const int b = blockIdx.y;
-  if (!active[b]) return;
-  const int nx = G.nx, ny = G.ny, ncell = G.ncell(), half = G.half();
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  const int col = t % tl.TX, rg = t / tl.TX;
-  const int bx = blockIdx.x % tl.ntx, by = blockIdx.x / tl.ntx;
-  const int i = bx * tl.TX + col;
-  const int j0 = by * tl.GR * tl.R + rg * tl.R;
-  const bool thr = rg < tl.GR && i < nx;
-  // where the east neighbour's state and the west face come from
-  const bool east_in = thr && col < tl.TX - 1 && i < nx - 1;   // a thread of this tile
-  const bool east_lane = east_in && lane < 31;
-  const bool east_smem = east_in && lane == 31;
-  const bool east_load = thr && col == tl.TX - 1 && i < nx - 1;  // tile edge
-  const bool west_in = thr && col > 0;
-  const bool west_lane = west_in && lane > 0;
-  const bool west_smem = west_in && lane == 0;
-  const bool west_load = thr && col == 0 && i > 0;               // tile edge
-  const int64_t o = (int64_t)b * ncell;
-  const double* pb_ = p + o;
-  const double* cb_ = c + o;
-  const double hd = 0.5 * P.drho;              // rho_bar = rho0 + hd (c_L + c_U)
-  const double hdg = hd * P.g * G.hy;          // gravity term of a vertical face: hdg (c_L + c_U)
-  // one face L -> U: mass and salt flux from both sides' p, c, rho, rho c
-  auto face = [&](double pL, double cL, double rL, double rcL, double pU, double cU, double rU,
-                  double rcU, double tf, double dco, bool vert, double& q, double& Fm,
-                  double& Fs) {
-    const double sc = cL + cU;
-    const double rbar = fma(hd, sc, P.rho0);
-    const double dp = pU - pL;
-    q = -tf * (vert ? fma(hdg, sc, dp) : dp);
-    const bool up = q >= 0.0;
-    Fm = q * (up ? rL : rU);
-    Fs = fma(q, up ? rcL : rcU, -(dco * rbar) * (cU - cL));
-  };
-  double v = 0.0;
-  double pP = 0.0, cP = 0.0, rP = 0.0, rcP = 0.0, FmS = 0.0, FsS = 0.0;
-  if (thr && j0 < ny) {
-    pP = pb_[j0 * nx + i];
-    cP = cb_[j0 * nx + i];
-  }
-  rP = fma(P.drho, cP, P.rho0);
-  rcP = rP * cP;
-  if (thr && j0 < ny && j0 > 0) {   // south face of the first row (every thread of a row group)
-    const int id = (j0 - 1) * nx + i;
-    const double pS = pb_[id], cS = cb_[id];
-    const double rS = fma(P.drho, cS, P.rho0);
-    double q;
-    face(pS, cS, rS, rS * cS, pP, cP, rP, rcP, ty[o + id], dy[o + id], true, q, FmS, FsS);
-  }
-  for (int r = 0; r < tl.R; ++r) {
-    const int j = j0 + r;
-    const bool cv = thr && j < ny;
-    const int id = j * nx + i;
-    // east neighbour: the next lane's state, across a warp edge through
-    // shared memory, at a tile edge from memory, at the right side the
-    // seawater values
-    if (lane == 0) { shS[0][w] = pP; shS[1][w] = cP; shS[2][w] = rP; shS[3][w] = rcP; }
-    double pE = __shfl_down_sync(0xffffffffu, pP, 1);
-    double cE = __shfl_down_sync(0xffffffffu, cP, 1);
-    double rE = __shfl_down_sync(0xffffffffu, rP, 1);
-    double rcE = __shfl_down_sync(0xffffffffu, rcP, 1);
-    __syncthreads();
-    if (east_smem) { pE = shS[0][w + 1]; cE = shS[1][w + 1]; rE = shS[2][w + 1]; rcE = shS[3][w + 1]; }
-    if (!east_lane && !east_smem) {
-      if (east_load && cv) {
-        pE = pb_[id + 1];
-        cE = cb_[id + 1];
-      } else {   // the right side: reduced seawater pressure at this row, c = 1
-        pE = P.drho * P.g * (P.Ly - (j + 0.5) * G.hy);
-        cE = 1.0;
-      }
-      rE = fma(P.drho, cE, P.rho0);
-      rcE = rE * cE;
-    }
-    double FmE = 0.0, FsE = 0.0, qE = 0.0;
-    if (cv) face(pP, cP, rP, rcP, pE, cE, rE, rcE, tx[o + id], dx[o + id], false, qE, FmE, FsE);
-    // west face: the previous lane's east face (across a warp edge through
-    // shared memory; recomputed at a tile edge)
-    if (lane == 31) { shF[0][w] = FmE; shF[1][w] = FsE; }
-    double FmW = __shfl_up_sync(0xffffffffu, FmE, 1);
-    double FsW = __shfl_up_sync(0xffffffffu, FsE, 1);
-    __syncthreads();
-    if (west_smem) { FmW = shF[0][w - 1]; FsW = shF[1][w - 1]; }
-    if (!west_in) { FmW = 0.0; FsW = 0.0; }
-    if (west_load && cv) {
-      const double pW = pb_[id - 1], cW = cb_[id - 1];
-      const double rW = fma(P.drho, cW, P.rho0);
-      double q;
-      face(pW, cW, rW, rW * cW, pP, cP, rP, rcP, tx[o + id - 1], dx[o + id - 1], false, q, FmW,
-           FsW);
-    }
-    double pN = 0.0, cN = 0.0;
-    double FmN = 0.0, FsN = 0.0, qN = 0.0;
-    if (cv && j < ny - 1) {
-      pN = pb_[id + nx];
-      cN = cb_[id + nx];
-    }
-    const double rN = fma(P.drho, cN, P.rho0);
-    const double rcN = rN * cN;
-    if (cv && j < ny - 1) face(pP, cP, rP, rcP, pN, cN, rN, rcN, ty[o + id], dy[o + id], true, qN, FmN, FsN);
-    if (cv) {
-      const double a = vt[o + id] * rP;
-      double Rp = (a - mo[o + id]) + FmE + FmN - FmW - FmS;
-      double Rc = fma(a, cP, -so[o + id]) + FsE + FsN - FsW - FsS;
-      if (i == 0) {   // left side: fresh-water inflow, diffusion to c = 0 at hx/2
-        Rp += -G.hy * P.rho0 * qin[(int64_t)b * ny + j];
-        Rc += ((2.0 * G.hy * P.D / G.hx) * phi[o + id]) * (0.5 * (rP + P.rho0)) * cP;
-      }
-      const int cs = cs_pos(i, j, nx, half);
-      const int64_t ob = (int64_t)b * 2 * ncell;
-      const T* Jb = J + (int64_t)b * kJP * ncell + cs;
-      const T mp = (T)(-Rp), mc = (T)(-Rc);
-      bvec[ob + cs] = Jb[0] * mp + Jb[(int64_t)ncell] * mc;
-      bvec[ob + ncell + cs] = Jb[(int64_t)2 * ncell] * mp + Jb[(int64_t)3 * ncell] * mc;
-      xvec[ob + cs] = (T)0;
-      xvec[ob + ncell + cs] = (T)0;
-      qx[o + id] = qE;
-      qy[o + id] = qN;
-      v = fma(Rp, Rp, fma(Rc, Rc, v));
-    }
-    FmS = FmN;
-    FsS = FsN;
-    pP = pN;
-    cP = cN;
-    rP = rN;
-    rcP = rcN;
-  }
-  const double s = block_sum(v, shr);
-  if (threadIdx.x == 0) partial[(int64_t)b * gridDim.x + blockIdx.x] = s;
-}
-
-// Per-sample convergence decision after k_resjac, one warp per sample:
+// Per-sample convergence decision after k_residual, one warp per sample:
 // sums the sample's partials in a fixed order, scales the RMS residual to
 // units of c per step, updates active / status / counters. A sample is
 // converged when r <= max(rtol r0, atol), or when r <= max(stag_tol,
@@ -1381,17 +1039,6 @@ k_qoi(unsigned long long* ctr, Phys P, Geom G, int B, const double* __restrict__
 #pragma unroll
     for (int m = 0; m < 15; ++m) qb[7 + m] = box[m];
   }
-}
-
-// p -> p' = p - rho0 g (Ly - y) for the natural-layout entry point.
-static __global__ void k_reduce_pressure(Phys P, Geom G, int B, const double* __restrict__ p,
-                                  double* __restrict__ pr) {
-  const int64_t n = (int64_t)B * G.ncell();
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n) return;
-  const int cell = (int)(idx % G.ncell());
-  const int j = cell / G.nx;
-  pr[idx] = p[idx] - P.rho0 * P.g * (P.Ly - (j + 0.5) * G.hy);
 }
 
 // ---------------------------------------------------------------------------

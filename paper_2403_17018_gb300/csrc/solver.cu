@@ -78,8 +78,12 @@ Solver::Solver(const henry_config& cfg, int nx, int ny, int nt) : cfg_(cfg), nt_
   build_hierarchy(nx, ny, cfg.Lx, cfg.Ly, geoms_);
   levels_.resize(geoms_.size());
   for (size_t k = 0; k < geoms_.size(); ++k) levels_[k].g = geoms_[k];
-  tile_ = make_res_tile(geoms_.back().nx, geoms_.back().ny, cfg.res_rows);
-  nchunk_ = tile_.ntx * tile_.nty;
+  const Geom& fine = geoms_.back();
+  // four columns per thread where the grid has warps to spare (see make_res_tile)
+  res_cols_ = fine.nx % 4 == 0 && fine.ncell() > 4096 ? 4 : 2;
+  tile_r_ = make_res_tile(fine.nx, fine.ny, res_cols_, cfg.res_rows, false);
+  tile_j_ = make_res_tile(fine.nx, fine.ny, 2, cfg.res_rows, true);
+  nchunk_ = cfg.jac_lag ? tile_r_.warps() : tile_j_.warps();
   ks_ = 0;
   kc_ = 0;
   for (size_t k = 0; k < geoms_.size(); ++k) {
@@ -250,6 +254,9 @@ int Solver::ensure(int B, cudaStream_t s) {
   const size_t o_mo = take((size_t)F.ncell() * Bz * 8);
   const size_t o_so = take((size_t)F.ncell() * Bz * 8);
   const size_t o_vt = take((size_t)F.ncell() * Bz * 8);
+  const size_t o_dxh = take((size_t)F.ncell() * Bz * 8);
+  const size_t o_dyh = take((size_t)F.ncell() * Bz * 8);
+  const size_t o_tf = take(tsize_ == sizeof(float) ? (size_t)F.ncell() * Bz * 16 : 0);
   const size_t o_step = take(8);
   const size_t o_qin = take((size_t)F.ny * Bz * 8);
   const size_t o_qin0 = take((size_t)F.ny * Bz * 8);
@@ -306,6 +313,9 @@ int Solver::ensure(int B, cudaStream_t s) {
   mo_ = (double*)(a + o_mo);
   so_ = (double*)(a + o_so);
   vt_ = (double*)(a + o_vt);
+  dxh_ = (double*)(a + o_dxh);
+  dyh_ = (double*)(a + o_dyh);
+  tf_ = tsize_ == sizeof(float) ? (float4*)(a + o_tf) : nullptr;
   step_ = (int*)(a + o_step);
   qin_ = (double*)(a + o_qin);
   qin0_ = (double*)(a + o_qin0);
@@ -556,10 +566,7 @@ template <typename T>
 void Solver::enqueue_rebuild(int B, cudaStream_t s) {
   const int* refresh = cfg_.jac_lag ? refresh_ : nullptr;
   if (refresh) {
-    MGLevel& F = levels_.back();
-    k_resjac<T, false><<<dim3(nchunk_, B), kBlock, 0, s>>>(
-        counter_, phys_, F.g, F.g.hx * F.g.hy / tau_, B, tile_, F.p, F.c, c_old_, F.phi, F.K, F.tx,
-        F.dx, F.ty, F.dy, qin_, active_, (T*)F.J, (T*)F.b, (T*)F.x, partial_, F.qx, F.qy, refresh);
+    launch_resjac<T>(B, refresh, nullptr, s);
   }
   enqueue_coarse_ops<T>(B, s, refresh);
   enqueue_coarse_inv<T>(B, s, refresh);
@@ -584,19 +591,63 @@ void Solver::enqueue_iteration(int B, cudaStream_t s) {
   enqueue_solve_update<T>(B, s);
 }
 
+// Inputs of k_residual on the finest level's workspace.
+ResArgs Solver::res_args() const {
+  const MGLevel& F = levels_.back();
+  ResArgs a = {};
+  a.p = F.p;
+  a.c = F.c;
+  a.c_old = c_old_;
+  a.phi = F.phi;
+  a.K = F.K;
+  a.tx = F.tx;
+  a.dx = dxh_;
+  a.ty = F.ty;
+  a.dy = dyh_;
+  a.tf = tf_;
+  a.qin = qin_;
+  a.vt = vt_;
+  a.mo = mo_;
+  a.so = so_;
+  a.active = active_;
+  a.qx = F.qx;
+  a.qy = F.qy;
+  return a;
+}
+
+// Residual only, with the operators of the last rebuild.
+template <typename T>
+void Solver::launch_resid(int B, cudaStream_t s) {
+  MGLevel& F = levels_.back();
+  ResArgs a = res_args();
+  a.partial = partial_;
+  auto kern = res_cols_ == 4 ? k_residual<T, 4, false, false, false, true>
+                             : k_residual<T, 2, false, false, false, true>;
+  kern<<<dim3(tile_r_.warps(), B), 32, 0, s>>>(counter_, phys_, F.g, F.g.hx * F.g.hy / tau_, tile_r_,
+                                               a, (T*)F.J, (T*)F.b, (T*)F.x);
+}
+
+// Residual and operators of the finest level, for the samples that ask for
+// them (refresh).
+template <typename T>
+void Solver::launch_resjac(int B, const int* refresh, double* partial, cudaStream_t s) {
+  MGLevel& F = levels_.back();
+  ResArgs a = res_args();
+  a.refresh = refresh;
+  a.partial = partial;
+  k_residual<T, 2, true, false, false, true><<<dim3(tile_j_.warps(), B), 32, 0, s>>>(counter_, phys_, F.g, F.g.hx * F.g.hy / tau_, tile_j_,
+                                               a, (T*)F.J, (T*)F.b, (T*)F.x);
+}
+
 template <typename T>
 void Solver::enqueue_resjac_check(int B, cudaStream_t s, bool set_cond,
                                   unsigned long long cond) {
   MGLevel& F = levels_.back();
   const Geom& G = F.g;
   if (cfg_.jac_lag)   // residual only; the next iteration rebuilds operators where needed
-    k_resid<T><<<dim3(nchunk_, B), kBlock, 0, s>>>(
-        counter_, phys_, G, B, tile_, F.p, F.c, vt_, mo_, so_, F.phi, F.tx, F.dx, F.ty, F.dy,
-        qin_, active_, (const T*)F.J, (T*)F.b, (T*)F.x, partial_, F.qx, F.qy);
+    launch_resid<T>(B, s);
   else
-    k_resjac<T, false><<<dim3(nchunk_, B), kBlock, 0, s>>>(
-        counter_, phys_, G, G.hx * G.hy / tau_, B, tile_, F.p, F.c, c_old_, F.phi, F.K, F.tx, F.dx,
-        F.ty, F.dy, qin_, active_, (T*)F.J, (T*)F.b, (T*)F.x, partial_, F.qx, F.qy, nullptr);
+    launch_resjac<T>(B, nullptr, partial_, s);
   int* refresh = cfg_.jac_lag ? refresh_ : nullptr;
   // residual scaled to units of c per step: RMS(R) * tau / (V phi0 rho0)
   const double scale = tau_ / (G.hx * G.hy * cfg_.phi0 * cfg_.rho0);
@@ -802,7 +853,8 @@ int Solver::setup_t(const double* xi, const double* logk, int B, cudaStream_t s)
   for (int k = 0; k < nl; ++k) {
     MGLevel& L = levels_[k];
     k_face_consts<<<grid1((int64_t)B * L.g.ncell()), kBlock, 0, s>>>(
-        counter_, phys_, L.g, B, L.phi, L.K, L.tx, L.dx, L.ty, L.dy);
+        counter_, phys_, L.g, B, L.phi, L.K, L.tx, L.dx, L.ty, L.dy, k == nl - 1 ? dxh_ : nullptr,
+        k == nl - 1 ? dyh_ : nullptr, k == nl - 1 ? tf_ : nullptr);
   }
   k_init_state<<<grid1((int64_t)B * G.ncell()), kBlock, 0, s>>>(counter_, phys_, G, B, F.p, F.c,
                                                                 iters_w_, step_);
@@ -897,13 +949,9 @@ void Solver::launch_timed(int which, int B, cudaStream_t s) {
     k_smooth<T><<<grid1((int64_t)B * F.g.half()), kBlock, 0, s>>>(
         counter_, F.g, B, 0, active_, (const T*)F.J, (const T*)F.b, (T*)F.x);
   } else if (which == 2) {
-    k_resid<T><<<dim3(nchunk_, B), kBlock, 0, s>>>(
-        counter_, phys_, F.g, B, tile_, F.p, F.c, vt_, mo_, so_, F.phi, F.tx, F.dx, F.ty, F.dy,
-        qin_, active_, (const T*)F.J, (T*)F.b, (T*)F.x, partial_, F.qx, F.qy);
+    launch_resid<T>(B, s);
   } else {
-    k_resjac<T, false><<<dim3(nchunk_, B), kBlock, 0, s>>>(
-        counter_, phys_, F.g, F.g.hx * F.g.hy / tau_, B, tile_, F.p, F.c, c_old_, F.phi, F.K, F.tx, F.dx, F.ty, F.dy,
-        qin_, active_, (T*)F.J, (T*)F.b, (T*)F.x, partial_, F.qx, F.qy, nullptr);
+    launch_resjac<T>(B, nullptr, nullptr, s);
   }
 }
 
@@ -1144,12 +1192,9 @@ int Solver::adjoint_t(const double* xi, const double* logk, int B, int qoi, int 
       CK(cudaMemcpyAsync(c_old_, uprev + n, n * 8, cudaMemcpyDeviceToDevice, s));
       k_activate<<<grid1(B), kBlock, 0, s>>>(counter_, B, status_w_, active_, it_step_);
       // operators of step st: J (multigrid type, every level) and exact FP64 J
-      k_resjac<T, false><<<dim3(nchunk_, B), kBlock, 0, s>>>(
-          counter_, phys_, G, G.hx * G.hy / tau_, B, tile_, F.p, F.c, c_old_, F.phi, F.K, F.tx, F.dx, F.ty, F.dy,
-          qin_, active_, (T*)F.J, (T*)F.b, (T*)F.x, partial_, F.qx, F.qy, nullptr);
-      k_resjac<double, true><<<dim3(nchunk_, B), kBlock, 0, s>>>(
-          counter_, phys_, G, G.hx * G.hy / tau_, B, tile_, F.p, F.c, c_old_, F.phi, F.K, F.tx, F.dx, F.ty, F.dy,
-          qin_, active_, J64_, res_, nullptr, nullptr, nullptr, nullptr, nullptr);
+      launch_resjac<T>(B, nullptr, nullptr, s);
+      k_residual<double, 2, true, true, false, true><<<dim3(tile_j_.warps(), B), 32, 0, s>>>(
+          counter_, phys_, G, G.hx * G.hy / tau_, tile_j_, res_args(), J64_, res_, nullptr);
       enqueue_coarse_ops<T>(B, s, nullptr);
       for (size_t k = 0; k < levels_.size(); ++k)
         k_transpose<T><<<grid1((int64_t)B * levels_[k].g.ncell()), kBlock, 0, s>>>(
@@ -1217,20 +1262,23 @@ int or_status(const int* src, int* dst, int B, unsigned long long* ctr, cudaStre
 cudaError_t launch_residual_jacobian(const Phys& P, const Geom& G, double tau, int B,
                                      const double* phi, const double* K, const double* qin,
                                      const double* p, const double* c, const double* c_old,
-                                     double* R, double* J, double* scratch, cudaStream_t s) {
-  const int64_t n = (int64_t)B * G.ncell();
-  const int grid = (int)((n + kBlock - 1) / kBlock);
-  double* tx = scratch;
-  double* dx = scratch + n;
-  double* ty = scratch + 2 * n;
-  double* dy = scratch + 3 * n;
-  double* pr = scratch + 4 * n;
-  k_face_consts<<<grid, kBlock, 0, s>>>(nullptr, P, G, B, phi, K, tx, dx, ty, dy);
-  k_reduce_pressure<<<grid, kBlock, 0, s>>>(P, G, B, p, pr);
-  const ResTile tl = make_res_tile(G.nx, G.ny);
-  k_resjac<double, true><<<dim3(tl.ntx * tl.nty, B), kBlock, 0, s>>>(
-      nullptr, P, G, G.hx * G.hy / tau, B, tl, pr, c, c_old, phi, K, tx, dx, ty, dy, qin, nullptr, J, R, nullptr,
-      nullptr, nullptr, nullptr, nullptr);
+                                     double* R, double* J, cudaStream_t s) {
+  ResArgs a = {};
+  a.p = p;
+  a.c = c;
+  a.c_old = c_old;
+  a.phi = phi;
+  a.K = K;
+  a.qin = qin;
+  // two columns per thread with 16-byte loads where every row allows them
+  const uintptr_t al = (uintptr_t)p | (uintptr_t)c | (uintptr_t)c_old | (uintptr_t)phi | (uintptr_t)K;
+  const bool two = G.nx % 2 == 0 && al % 16 == 0;
+  const ResTile t = make_res_tile(G.nx, G.ny, two ? 2 : 1, 0, true);
+  auto kern = two ? (J ? k_residual<double, 2, true, true, true, true>
+                       : k_residual<double, 2, false, true, true, true>)
+                  : (J ? k_residual<double, 1, true, true, true, false>
+                       : k_residual<double, 1, false, true, true, false>);
+  kern<<<dim3(t.warps(), B), 32, 0, s>>>(nullptr, P, G, G.hx * G.hy / tau, t, a, J, R, nullptr);
   return cudaGetLastError();
 }
 

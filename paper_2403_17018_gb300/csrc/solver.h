@@ -126,6 +126,10 @@ class Solver {
   template <typename T> int capture_body_t(const StepBody& sb, int B, cudaStream_t bs);
   template <typename T> int step_graph(int B, cudaStream_t s);
   template <typename T> void launch_timed(int which, int B, cudaStream_t s);
+  ResArgs res_args() const;
+  template <typename T> void launch_resid(int B, cudaStream_t s);
+  template <typename T> void launch_resjac(int B, const int* refresh, double* partial,
+                                           cudaStream_t s);
   template <typename T> void launch_small(int B, int ncycles, cudaStream_t s);
   template <typename T> void launch_cluster(int B, int ncycles, cudaStream_t s);
   int ensure(int B, cudaStream_t s);
@@ -159,9 +163,11 @@ class Solver {
   // state components per adjoint checkpoint: u, u^(n-1) and the older
   // states of the guess
   size_t ckpt_width() const { return 4 + 2 * (size_t)guess_depth(); }
-  double* mo_ = nullptr;        // old-time storage terms of the step (k_resid)
+  double* mo_ = nullptr;        // old-time storage terms of the step (k_residual)
   double* so_ = nullptr;
-  double* vt_ = nullptr;        // V phi / tau per cell (k_resid)
+  double* vt_ = nullptr;        // V phi / tau per cell (k_residual)
+  double *dxh_ = nullptr, *dyh_ = nullptr;   // halves of the finest dx, dy (k_residual)
+  float4* tf_ = nullptr;        // FP32 face constants of the finest level (FP32 multigrid)
   int* step_ = nullptr;         // completed steps of the current solve (device)
   double* qin_ = nullptr;
   double* qin0_ = nullptr;     // inflow base of the paper field model (time factor per step)
@@ -186,8 +192,9 @@ class Solver {
   unsigned long long* counter_ = nullptr;  // device launch counter
   int prio_ = 0;
   int* keep_ = nullptr;       // device flag: operators kept across steps (k_check)
-  int nchunk_ = 0;            // residual blocks per sample
-  ResTile tile_{};            // tiling of the residual kernel
+  int nchunk_ = 0;            // residual partial sums per sample (k_check)
+  int res_cols_ = 2;          // columns per thread of the residual-only kernel
+  ResTile tile_r_{}, tile_j_{};   // tiling of k_residual without and with the Jacobian
   int ks_ = 0;                // top multigrid level handled by k_vcycle_small
   int kc_ = 0;                // top multigrid level handled by k_vcycle_cluster
   int cl_ = 1;                // blocks per cluster (one cluster per sample)
