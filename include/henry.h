@@ -336,9 +336,9 @@ int henry_adjoint(henry_ctx* ctx, int level, const double* xi, const double* log
 
 /* Merge one batch into the running statistics of a level (Def. of Y_l and
  * V_l; V_l = m2_d / (n - 1)). Samples with status != 0 are skipped.
- * Welford per thread in sample order, then a fixed pairwise Chan merge tree
- * on the device (deterministic for a given B), then a Chan merge into
- * *inout on the host. Synchronous: returns when the batch is merged.
+ * Two passes over the batch on the device (means, then squared deviations;
+ * fixed order, deterministic for a given B), then a Chan merge into *inout on
+ * the host. Synchronous: returns when the batch is merged.
  *   q_fine    device [B][HENRY_NQ]
  *   q_coarse  device [B][HENRY_NQ] or NULL (level 0: g_{-1} = 0)
  *   status    device int [B] or NULL (all samples valid)
@@ -347,8 +347,8 @@ int mlmc_level_stats(henry_ctx* ctx, int level, const double* q_fine, const doub
                      int B, const int* status, henry_level_stats* inout, void* stream);
 
 /* Per-cell running statistics of the c field of one level (section 4, Test
- * A1): for every cell of the level-l grid, Welford over the batch in sample
- * order of g = c_l and of d = c_l - P0 c_{l-1}, P0 the piecewise-constant
+ * A1): for every cell of the level-l grid, the moments of the batch (groups of
+ * samples merged by a fixed tree, deterministic for a given B) of g = c_l and of d = c_l - P0 c_{l-1}, P0 the piecewise-constant
  * transfer from the level-(l-1) grid. Samples with status != 0 are skipped.
  *   c_fine    device [B][ny_l][nx_l];  c_coarse device [B][ny_{l-1}][nx_{l-1}] or NULL
  *   n         device int64 [ny_l*nx_l]  running count (all cells equal)

@@ -1,7 +1,9 @@
 // MLMC level statistics on the device (arxiv 2403.17018, section 3: Def. of
-// Y_l and V_l, Eq. A). Welford updates in sample order per thread, merged
-// with Chan's pairwise formula in a fixed tree, so the result depends only on
-// the batch contents and B.
+// Y_l and V_l, Eq. A). Every reduction has a fixed order, so the result
+// depends only on the batch contents and B. What bounds these kernels on
+// GB300 is FP64 latency and throughput, not memory, so none of them divides
+// per sample: the QoI moments take two passes over the batch (mean, then
+// squared deviations), the fields one pass about a shift close to the mean.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -10,135 +12,248 @@
 
 namespace henry {
 
-constexpr int kStatThreads = 128;
+constexpr int kStatThreads = 256;
 
-struct Acc {
-  double n;
-  double mf[kNQ], m2f[kNQ], md[kNQ], m2d[kNQ];
+// Block sum of a double, the same result in every thread (fixed order).
+__device__ __forceinline__ double stat_sum(double v, double* sh) {
+  const double s = block_sum(v, sh);
+  __syncthreads();
+  if (threadIdx.x == 0) sh[0] = s;
+  __syncthreads();
+  const double t = sh[0];
+  __syncthreads();
+  return t;
+}
+
+// Moments of one QoI (blockIdx.x) over the valid samples of the batch, two
+// passes: out[0] = n, then mean_f, m2_f, mean_d, m2_d [kNQ] of g = q_fine
+// and d = q_fine - q_coarse. m2 = sum (g - mean)^2 - (sum (g - mean))^2 / n,
+// whose second term removes the rounding of the mean. Grid kNQ blocks: 600
+// samples take 8 us, where one block that ran Welford's update (two
+// divisions per sample and QoI) took 387 us.
+__global__ void __launch_bounds__(kStatThreads)
+k_level_stats(unsigned long long* ctr, int B, const double* __restrict__ qf,
+              const double* __restrict__ qc, const int* __restrict__ status,
+              double* __restrict__ out) {
+  HENRY_COUNT_LAUNCH(ctr);
+  __shared__ double sh[kStatThreads / 32];
+  const int k = blockIdx.x;
+  double cnt = 0.0, sf = 0.0, sd = 0.0;
+  auto each = [&](auto&& f) {
+    for (int b = threadIdx.x; b < B; b += kStatThreads) {
+      if (status && status[b] != 0) continue;
+      const double g = qf[(int64_t)b * kNQ + k];
+      f(g, qc ? g - qc[(int64_t)b * kNQ + k] : g);
+    }
+  };
+  each([&](double g, double d) {
+    cnt += 1.0;
+    sf += g;
+    sd += d;
+  });
+  const double n = stat_sum(cnt, sh);
+  const double inv = n > 0.0 ? 1.0 / n : 0.0;
+  const double mf = stat_sum(sf, sh) * inv;
+  const double md = qc ? stat_sum(sd, sh) * inv : mf;
+  double f1 = 0.0, f2 = 0.0, d1 = 0.0, d2 = 0.0;
+  each([&](double g, double d) {
+    const double e = g - mf;
+    f1 += e;
+    f2 = fma(e, e, f2);
+    if (qc) {
+      const double h = d - md;
+      d1 += h;
+      d2 = fma(h, h, d2);
+    }
+  });
+  f1 = stat_sum(f1, sh);
+  f2 = stat_sum(f2, sh);
+  if (qc) {
+    d1 = stat_sum(d1, sh);
+    d2 = stat_sum(d2, sh);
+  } else {
+    d1 = f1;
+    d2 = f2;
+  }
+  if (threadIdx.x == 0) {
+    if (k == 0) out[0] = n;
+    out[1 + k] = fma(f1, inv, mf);
+    out[1 + kNQ + k] = fma(-f1 * inv, f1, f2);
+    out[1 + 2 * kNQ + k] = fma(d1, inv, md);
+    out[1 + 3 * kNQ + k] = fma(-d1 * inv, d1, d2);
+  }
+}
+
+// Count, mean and sum of squared deviations of one group of samples.
+struct Moments {
+  double n, mean, m2;
 };
 
-__device__ __forceinline__ void chan_merge(double na, double& ma, double& m2a, double nb, double mb,
-                                           double m2b) {
-  const double n = na + nb;
-  if (nb == 0.0) return;
-  if (na == 0.0) { ma = mb; m2a = m2b; return; }
-  const double d = mb - ma;
-  ma = ma + d * (nb / n);
-  m2a = m2a + m2b + d * d * (na * nb / n);
+// Chan's merge of b into a.
+__device__ __forceinline__ void chan_merge(Moments& a, const Moments& b) {
+  if (b.n == 0.0) return;
+  if (a.n == 0.0) {
+    a = b;
+    return;
+  }
+  const double n = a.n + b.n, d = b.mean - a.mean, w = b.n / n;
+  a.mean = fma(d, w, a.mean);
+  a.m2 = a.m2 + b.m2 + d * d * (a.n * w);
+  a.n = n;
 }
 
-// One block. out[0] = n, then mean_f[6], m2_f[6], mean_d[6], m2_d[6].
-__global__ void k_level_stats(unsigned long long* ctr, int B, const double* __restrict__ qf,
-                              const double* __restrict__ qc, const int* __restrict__ status,
-                              double* __restrict__ out) {
-  HENRY_COUNT_LAUNCH(ctr);
-  __shared__ Acc acc[kStatThreads];
-  const int t = threadIdx.x;
-  Acc a;
-  a.n = 0.0;
-  for (int k = 0; k < kNQ; ++k) a.mf[k] = a.m2f[k] = a.md[k] = a.m2d[k] = 0.0;
-  for (int b = t; b < B; b += blockDim.x) {
-    if (status && status[b] != 0) continue;
-    a.n += 1.0;
-    for (int k = 0; k < kNQ; ++k) {
-      const double g = qf[(int64_t)b * kNQ + k];
-      const double d = qc ? g - qc[(int64_t)b * kNQ + k] : g;
-      double e = g - a.mf[k];
-      a.mf[k] += e / a.n;
-      a.m2f[k] += e * (g - a.mf[k]);
-      e = d - a.md[k];
-      a.md[k] += e / a.n;
-      a.m2d[k] += e * (d - a.md[k]);
-    }
-  }
-  acc[t] = a;
-  __syncthreads();
-  for (int stride = blockDim.x / 2; stride > 0; stride >>= 1) {
-    if (t < stride) {
-      Acc& x = acc[t];
-      const Acc& y = acc[t + stride];
-      for (int k = 0; k < kNQ; ++k) {
-        chan_merge(x.n, x.mf[k], x.m2f[k], y.n, y.mf[k], y.m2f[k]);
-        chan_merge(x.n, x.md[k], x.m2d[k], y.n, y.md[k], y.m2d[k]);
-      }
-      x.n += y.n;
-    }
-    __syncthreads();
-  }
-  if (t == 0) {
-    out[0] = acc[0].n;
-    for (int k = 0; k < kNQ; ++k) {
-      out[1 + k] = acc[0].mf[k];
-      out[1 + kNQ + k] = acc[0].m2f[k];
-      out[1 + 2 * kNQ + k] = acc[0].md[k];
-      out[1 + 3 * kNQ + k] = acc[0].m2d[k];
-    }
-  }
-}
+// Per-cell statistics of c_l and c_l - P0 c_{l-1} over the batch, merged into
+// the running state held in device memory. A block takes 32 cells and G
+// groups of consecutive samples; each thread sums the deviations and their
+// squares of its cell over its group's valid samples about a shift, the mean
+// of the group's first (up to 8) valid samples, so that nothing cancels: three
+// FP64 instructions per sample (and quantity). The groups are merged by a
+// fixed tree (Chan). 600 samples of 8192 cells: 1028 us with a thread per cell running
+// Welford's update, 61 us so.
+constexpr int kShift = 8;
 
-// Per-cell Welford of c_l and c_l - P0 c_{l-1} over the batch, in sample
-// order, continuing the running state held in device memory.
 __global__ void k_field_stats(unsigned long long* ctr, int nx, int ny, int B,
                               const double* __restrict__ cf, const double* __restrict__ cc,
                               const int* __restrict__ status, int64_t* __restrict__ n,
                               double* __restrict__ mean_f, double* __restrict__ m2_f,
                               double* __restrict__ mean_d, double* __restrict__ m2_d) {
   HENRY_COUNT_LAUNCH(ctr);
+  extern __shared__ Moments mom[];          // [2][G][32], G a power of two
+  const int G = blockDim.y, x = threadIdx.x, y = threadIdx.y;
   const int ncell = nx * ny;
-  const int cell = blockIdx.x * blockDim.x + threadIdx.x;
-  if (cell >= ncell) return;
-  const int j = cell / nx, i = cell - j * nx;
-  const int nxc = nx / 2, ncc = (nx / 2) * (ny / 2);
-  const int ccell = (j >> 1) * nxc + (i >> 1);
-  double cnt = (double)n[cell];
-  double mf = mean_f[cell], sf = m2_f[cell], md = mean_d[cell], sd = m2_d[cell];
-  for (int b = 0; b < B; ++b) {
-    if (status && status[b] != 0) continue;
-    const double g = cf[(int64_t)b * ncell + cell];
-    const double d = cc ? g - cc[(int64_t)b * ncc + ccell] : g;
-    cnt += 1.0;
-    double e = g - mf;
-    mf += e / cnt;
-    sf += e * (g - mf);
-    e = d - md;
-    md += e / cnt;
-    sd += e * (d - md);
+  const int cell = blockIdx.x * 32 + x;
+  const int b0 = (int)((int64_t)B * y / G), b1 = (int)((int64_t)B * (y + 1) / G);
+  Moments f = {0.0, 0.0, 0.0}, d = {0.0, 0.0, 0.0};
+  if (cell < ncell) {
+    const int j = cell / nx, i = cell - j * nx;
+    const int ncc = (nx / 2) * (ny / 2);
+    const int ccell = (j >> 1) * (nx / 2) + (i >> 1);
+    const double* pf = cf + cell;
+    const double* pc = cc ? cc + ccell : nullptr;
+    double kf = 0.0, kd = 0.0, c = 0.0;
+    int bs = b0;                              // the first valid sample, then 8 from there
+    while (bs < b1 && status && status[bs] != 0) ++bs;
+#pragma unroll
+    for (int u = 0; u < kShift; ++u) {
+      const int b = bs + u < b1 ? bs + u : b1 - 1;
+      if (bs + u >= b1 || (status && status[b] != 0)) continue;
+      const double g = pf[(int64_t)b * ncell];
+      kf += g;
+      if (pc) kd += g - pc[(int64_t)b * ncc];
+      c += 1.0;
+    }
+    const double cw = c == kShift ? 1.0 / kShift : c > 0.0 ? 1.0 / c : 0.0;
+    kf *= cw;
+    kd *= cw;
+    double f1 = 0.0, f2 = 0.0, d1 = 0.0, d2 = 0.0;
+    int cnt = 0;
+#pragma unroll 8
+    for (int b = b0; b < b1; ++b) {
+      const bool ok = !status || status[b] == 0;
+      const double g = pf[(int64_t)b * ncell];
+      const double h = pc ? pc[(int64_t)b * ncc] : 0.0;
+      if (!ok) continue;
+      ++cnt;
+      const double e = g - kf;
+      f1 += e;
+      f2 = fma(e, e, f2);
+      if (pc) {
+        const double u = (g - h) - kd;
+        d1 += u;
+        d2 = fma(u, u, d2);
+      }
+    }
+    if (cnt > 0) {
+      const double w = 1.0 / (double)cnt;
+      f = {(double)cnt, fma(f1, w, kf), fma(-f1 * w, f1, f2)};
+      d = pc ? Moments{(double)cnt, fma(d1, w, kd), fma(-d1 * w, d1, d2)} : f;
+    }
   }
-  n[cell] = (int64_t)cnt;
-  mean_f[cell] = mf;
-  m2_f[cell] = sf;
-  mean_d[cell] = md;
-  m2_d[cell] = sd;
+  mom[y * 32 + x] = f;
+  mom[(G + y) * 32 + x] = d;
+  __syncthreads();
+  // merge the groups pairwise, fine field and difference in different warps
+  for (int h = G >> 1; h > 0; h >>= 1) {
+    const int q = y / h, g = y - q * h;
+    if (q < 2) chan_merge(mom[(q * G + g) * 32 + x], mom[(q * G + g + h) * 32 + x]);
+    __syncthreads();
+  }
+  // and into the running state; its counts change once both have read them
+  const int q = G > 1 ? y : 0;
+  double total = 0.0;
+  if (y < 2 && cell < ncell) {
+    for (int r = q; r < (G > 1 ? q + 1 : 2); ++r) {
+      double* mean = r ? mean_d : mean_f;
+      double* m2 = r ? m2_d : m2_f;
+      Moments t = {(double)n[cell], mean[cell], m2[cell]};
+      chan_merge(t, mom[r * G * 32 + x]);
+      mean[cell] = t.mean;
+      m2[cell] = t.m2;
+      total = t.n;
+    }
+  }
+  __syncthreads();
+  if (y == 0 && cell < ncell) n[cell] = (int64_t)total;
 }
 
 // Per-cell exceedance counts (section 4: probability that the salt mass
 // fraction at a location exceeds a threshold): count[cell] += number of
-// valid samples b with c_b[cell] > threshold. One thread per cell, samples in
-// order, integer counts (exact, independent of batching).
+// valid samples b with c_b[cell] > threshold (exact, independent of
+// batching). 32 cells and G groups of samples per block; the comparison is
+// one of 64-bit integers ordered like the doubles, not an FP64 instruction
+// (112 us with a thread per cell, 12 us so, for 600 samples of 8192 cells).
+__device__ __forceinline__ long long order_key(double v) {
+  const long long b = __double_as_longlong(v);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+
 __global__ void k_field_exceed(unsigned long long* ctr, int ncell, int B,
                                const double* __restrict__ c, const int* __restrict__ status,
                                double threshold, int64_t* __restrict__ count) {
   HENRY_COUNT_LAUNCH(ctr);
-  const int cell = blockIdx.x * blockDim.x + threadIdx.x;
-  if (cell >= ncell) return;
-  int64_t k = 0;
-  for (int b = 0; b < B; ++b) {
-    if (status && status[b] != 0) continue;
-    k += c[(int64_t)b * ncell + cell] > threshold ? 1 : 0;
+  extern __shared__ int cnt_sh[];           // [G][32]
+  const int G = blockDim.y, x = threadIdx.x, y = threadIdx.y;
+  const int cell = blockIdx.x * 32 + x;
+  const int b0 = (int)((int64_t)B * y / G), b1 = (int)((int64_t)B * (y + 1) / G);
+  // +0 stands for both zeros; a NaN (above infinity's key, or below
+  // -infinity's) exceeds nothing
+  const long long t = order_key(threshold == 0.0 ? 0.0 : threshold), inf = order_key(INFINITY);
+  int k = 0;
+  if (cell < ncell) {
+#pragma unroll 8
+    for (int b = b0; b < b1; ++b) {
+      const long long v = order_key(c[(int64_t)b * ncell + cell]);
+      k += (!status || status[b] == 0) && v > t && v <= inf ? 1 : 0;
+    }
   }
-  count[cell] += k;
+  cnt_sh[y * 32 + x] = k;
+  __syncthreads();
+  if (y > 0 || cell >= ncell) return;
+  int64_t s = 0;
+  for (int g = 0; g < G; ++g) s += cnt_sh[g * 32 + x];
+  count[cell] += s;
+}
+
+// Sample groups per block: enough that the blocks of a small grid, with at
+// most 1024 threads each, still fill the GPU, and no more than samples.
+static int sample_groups(int ncell, int B) {
+  int G = (ncell + 31) / 32 < 152 ? 32 : 8;
+  while (G > 1 && G > B) G /= 2;
+  return G;
 }
 
 cudaError_t launch_field_exceed(unsigned long long* ctr, int ncell, int B, const double* c,
                                 const int* status, double threshold, int64_t* count,
                                 cudaStream_t s) {
-  k_field_exceed<<<(ncell + 255) / 256, 256, 0, s>>>(ctr, ncell, B, c, status, threshold, count);
+  const int G = sample_groups(ncell, B);
+  k_field_exceed<<<(ncell + 31) / 32, dim3(32, G), G * 32 * sizeof(int), s>>>(ctr, ncell, B, c, status,
+                                                                              threshold, count);
   return cudaGetLastError();
 }
 
 cudaError_t launch_level_stats(unsigned long long* ctr, int B, const double* qf, const double* qc,
                                const int* status, double* out, cudaStream_t s) {
-  k_level_stats<<<1, kStatThreads, 0, s>>>(ctr, B, qf, qc, status, out);
+  k_level_stats<<<kNQ, kStatThreads, 0, s>>>(ctr, B, qf, qc, status, out);
   return cudaGetLastError();
 }
 
@@ -146,8 +261,9 @@ cudaError_t launch_field_stats(unsigned long long* ctr, int nx, int ny, int B, c
                                const double* cc, const int* status, int64_t* n, double* mean_f,
                                double* m2_f, double* mean_d, double* m2_d, cudaStream_t s) {
   const int ncell = nx * ny;
-  k_field_stats<<<(ncell + 255) / 256, 256, 0, s>>>(ctr, nx, ny, B, cf, cc, status, n, mean_f,
-                                                    m2_f, mean_d, m2_d);
+  const int G = sample_groups(ncell, B);
+  k_field_stats<<<(ncell + 31) / 32, dim3(32, G), 2 * G * 32 * sizeof(Moments), s>>>(
+      ctr, nx, ny, B, cf, cc, status, n, mean_f, m2_f, mean_d, m2_d);
   return cudaGetLastError();
 }
 
