@@ -351,163 +351,173 @@ __global__ void k_check(unsigned long long* ctr, int B, int nchunk, int ncell,
   }
 }
 
-// Linearisation point of level k-1 from level k: c averaged over the four
-// children, face fluxes summed over the two fine faces that make up each
-// coarse face (east faces of the right children, north faces of the top
-// children; at the right side these are the boundary fluxes). Linearising
-// every level about the same flux field keeps the upwind decisions of the
-// coarse operators consistent with the finest one.
-static __global__ void k_restrict_state(unsigned long long* ctr, Geom Gf, Geom Gc, int B,
-                                 const int* __restrict__ active, const double* __restrict__ cf,
-                                 const double* __restrict__ qxf, const double* __restrict__ qyf,
-                                 double* __restrict__ cc, double* __restrict__ qxc,
-                                 double* __restrict__ qyc, const int* __restrict__ refresh) {
-  HENRY_COUNT_LAUNCH(ctr);
-  const int64_t n = (int64_t)B * Gc.ncell();
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n) return;
-  const int b = (int)(idx / Gc.ncell());
-  if (!active[b] || (refresh && !refresh[b])) return;
-  const int cell = (int)(idx - (int64_t)b * Gc.ncell());
-  const int J = cell / Gc.nx, I = cell - J * Gc.nx;
-  const int nx = Gf.nx;
-  const int64_t f0 = (int64_t)b * Gf.ncell() + (2 * J) * nx + 2 * I;
-  cc[idx] = 0.25 * (cf[f0] + cf[f0 + 1] + cf[f0 + nx] + cf[f0 + nx + 1]);
-  qxc[idx] = qxf[f0 + 1] + qxf[f0 + nx + 1];
-  qyc[idx] = qyf[f0 + nx] + qyf[f0 + nx + 1];
-}
+// Coarse operators of a defect correction: the linearisation points of every
+// multigrid level below the finest (k_restrict_states), then every coarse
+// operator and the inverse of the coarsest (k_coarse_ops). One launch each:
+// level by level they were two launches per level plus one, each about as
+// long as its chain of dependent FP64 instructions and L2 reads whatever the
+// level's size (16 samples of the 64x32 hierarchy, FP64: 76 us per rebuild;
+// 128x64 x 64, FP32: 87 us).
+constexpr int kMaxLevels = 12;
 
-// Jacobian of a coarse multigrid level from its own state and fields.
-template <typename T>
-__global__ void __launch_bounds__(kBlock)
-k_jac(unsigned long long* ctr, Phys P, Geom G, double vtau, int B, const int* __restrict__ active,
-      const double* __restrict__ p, const double* __restrict__ c, const double* __restrict__ phi,
-      const double* __restrict__ K, const double* __restrict__ tx, const double* __restrict__ dx,
-      const double* __restrict__ ty, const double* __restrict__ dy, const double* __restrict__ qx,
-      const double* __restrict__ qy, T* __restrict__ J, const int* __restrict__ refresh) {
+struct CoarseStates {
+  int nl;                           // levels; the finest is nl - 1
+  Geom g[kMaxLevels];
+  double* c[kMaxLevels];
+  double* qx[kMaxLevels];
+  double* qy[kMaxLevels];
+};
+
+constexpr int kRestrictDepth = 5;   // levels that one launch descends
+
+// Linearisation points of levels top-1, ..., top-depth from level top: c
+// averaged over the four children, face fluxes summed over the two fine
+// faces that make up each coarse face (east faces of the right children,
+// north faces of the top children; at the right side these are the boundary
+// fluxes). Linearising every level about the same flux field keeps the upwind
+// decisions of the coarse operators consistent with the finest one. A tile of
+// W x W cells of level top-1, W = 2^(depth-1), descends to one cell; a block
+// takes kBlock / W^2 tiles, a cell of level top-1 per thread.
+static __global__ void __launch_bounds__(kBlock)
+k_restrict_states(unsigned long long* ctr, const __grid_constant__ CoarseStates M, int top, int depth,
+                  int B, const int* __restrict__ active, const int* __restrict__ refresh) {
   HENRY_COUNT_LAUNCH(ctr);
-  const int ncell = G.ncell();
-  const int64_t n = (int64_t)B * ncell;
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n) return;
-  const int b = (int)(idx / ncell);
-  if (!active[b] || (refresh && !refresh[b])) return;
-  const int cell = (int)(idx - (int64_t)b * ncell);
-  const int j = cell / G.nx, i = cell - j * G.nx;
-  const int64_t o = (int64_t)b * ncell;
-  CellIn in;
-  gather_cell(G, i, j, p + o, c + o, phi + o, K + o, tx + o, dx + o, ty + o, dy + o, in);
-  in.c_old = in.c;
-  in.qin = 0.0;
-  const int id = cell;
-  in.qE = qx[o + id];
-  in.qN = in.hasN ? qy[o + id] : 0.0;
-  in.qW = in.hasW ? qx[o + id - 1] : 0.0;
-  in.qS = in.hasS ? qy[o + id - G.nx] : 0.0;
-  double Rp, Rc;
-  T Jc[20];
-  cell_residual<T, true, true>(P, G, vtau, in, Rp, Rc, Jc);
-  T* Jb = J + (int64_t)b * kJP * ncell + cs_pos(i, j, G.nx, G.half());
-  T d[4];
-  store_operator<T>(Jb, ncell, Jc, d);
+  __shared__ double sc[kBlock], sx[kBlock], sy[kBlock];
+  const int lw = depth - 1, W = 1 << lw;
+  const Geom Gf = M.g[top], Gc = M.g[top - 1];
+  const int tpx = Gc.nx >> lw, tiles = tpx * (Gc.ny >> lw);
+  const int t = threadIdx.x;
+  const int64_t tile = (int64_t)blockIdx.x * (kBlock >> (2 * lw)) + (t >> (2 * lw));
+  const int b = (int)(tile / tiles);
+  bool on = b < B;
+  if (on) on = active[b] && (!refresh || refresh[b]);
+  const int tl = (int)(tile - (int64_t)b * tiles), ty = tl / tpx, tx = tl - ty * tpx;
+  const int u = t & ((W << lw) - 1);        // cell within the tile
+  int iy = u >> lw, ix = u & (W - 1);
+  double c = 0.0, qx = 0.0, qy = 0.0;
+  if (on) {
+    const int I = (tx << lw) + ix, J = (ty << lw) + iy;
+    const int nx = Gf.nx;
+    const int64_t f0 = (int64_t)b * Gf.ncell() + (2 * J) * nx + 2 * I;
+    const double *cf = M.c[top], *qxf = M.qx[top], *qyf = M.qy[top];
+    c = 0.25 * (cf[f0] + cf[f0 + 1] + cf[f0 + nx] + cf[f0 + nx + 1]);
+    qx = qxf[f0 + 1] + qxf[f0 + nx + 1];
+    qy = qyf[f0 + nx] + qyf[f0 + nx + 1];
+    const int64_t o = (int64_t)b * Gc.ncell() + J * Gc.nx + I;
+    M.c[top - 1][o] = c;
+    M.qx[top - 1][o] = qx;
+    M.qy[top - 1][o] = qy;
+  }
+  sc[t] = c;
+  sx[t] = qx;
+  sy[t] = qy;
+  const int base = t - u;                   // the tile's first entry
+  for (int d = 2; d <= depth; ++d) {
+    __syncthreads();
+    const int lv = depth - d, Wd = 1 << lv; // cells of the tile per side on level top-d
+    const bool mine = on && u < (Wd << lv);
+    iy = u >> lv;
+    ix = u & (Wd - 1);
+    if (mine) {
+      const int w = Wd << 1, f = base + 2 * iy * w + 2 * ix;
+      c = 0.25 * (sc[f] + sc[f + 1] + sc[f + w] + sc[f + w + 1]);
+      qx = sx[f + 1] + sx[f + w + 1];
+      qy = sy[f + w] + sy[f + w + 1];
+    }
+    __syncthreads();
+    if (mine) {
+      sc[t] = c;
+      sx[t] = qx;
+      sy[t] = qy;
+      const Geom G = M.g[top - d];
+      const int64_t o = (int64_t)b * G.ncell() + ((ty << lv) + iy) * G.nx + (tx << lv) + ix;
+      M.c[top - d][o] = c;
+      M.qx[top - d][o] = qx;
+      M.qy[top - d][o] = qy;
+    }
+  }
 }
 
 // Explicit inverse of the coarsest system (the direct coarse solve of the
-// multigrid, section 2.3), one block per sample: in-place Gauss-Jordan
-// elimination with partial pivoting by rows. Per pivot k, three phases
-// separated by barriers: warp 0 picks the pivot row and records the
-// multipliers of column k, the pivot row is swapped in and divided by the
-// pivot, and every other element is updated by its own thread. The column
-// interchanges that undo the row pivots (last pivot first) are folded into
-// the output index. Unknown order 2*cell + var, cell natural; the inverse is
-// stored transposed, Ainv^T[v][u] at v*n + u, so that the coarse solve
-// x = Ainv b reads it with lanes over u. The arithmetic is the multigrid
-// type T (the coarse solve is part of the preconditioner): one n^3
-// elimination per operator rebuild turns each coarse solve into one
-// parallel matrix-vector product instead of 2n dependent substitution
-// steps. Shared memory (dynamic): coarse_inv_smem_bytes<T>(n).
+// multigrid, section 2.3) by one block: Gauss-Jordan elimination with partial
+// pivoting by rows, one barrier per pivot. Every warp finds the pivot row and
+// the pivot's reciprocal for itself, and every element of the next matrix is
+// formed from the last one's in another buffer: row k and the pivot row
+// interchanged, the new row k divided by the pivot (its own column becoming 1
+// / pivot), f times it subtracted from the others (their column k becoming -f
+// / pivot). The column interchanges that undo the row pivots (last pivot
+// first) are folded into the output index. Unknown order 2*cell + var, cell
+// natural; the inverse is stored transposed, Ainv^T[v][u] at v*n + u, so that
+// the coarse solve x = Ainv b reads it with lanes over u. The arithmetic is
+// the multigrid type T (the coarse solve is part of the preconditioner): one
+// n^3 elimination per operator rebuild turns each coarse solve into one
+// parallel matrix-vector product instead of 2n dependent substitution steps.
+// Bound by the chain of n reciprocals and multiply-adds.
+constexpr int kInvThreads = 128;
+
 template <typename T>
 __host__ __device__ inline size_t coarse_inv_smem_bytes(int n) {
-  return ((size_t)n * (n + 1) + n + 2) * sizeof(T) + 2 * (size_t)n * sizeof(int);
+  return 2 * (size_t)n * (n + 1) * sizeof(T) + 2 * (size_t)n * sizeof(int);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kBlock)
-k_coarse_inv(unsigned long long* ctr, Geom G, int B, const int* __restrict__ active,
-             const T* __restrict__ J, T* __restrict__ AinvT, const int* __restrict__ refresh) {
-  HENRY_COUNT_LAUNCH(ctr);
-  extern __shared__ __align__(16) unsigned char inv_sh[];
-  const int b = blockIdx.x;
-  if (!active[b] || (refresh && !refresh[b])) return;
+__device__ __forceinline__ void coarse_inverse(const Geom& G, const T* Jb, T* __restrict__ out,
+                                               unsigned char* smem) {
   const int nc = G.ncell(), n = 2 * nc, half = G.half(), ld = n + 1;
-  T* A = (T*)inv_sh;
-  T* fcol = A + n * ld;                 // multipliers of column k, after the swap
-  T* rinv_sh = fcol + n;                // 1 / pivot
-  int* pv = (int*)(rinv_sh + 2);        // pivot row of each step
+  T* A = (T*)smem;
+  T* Y = A + n * ld;
+  int* pv = (int*)(Y + n * ld);         // pivot row of each step
   int* qcol = pv + n;                   // output column -> eliminated column
   const int l = threadIdx.x & 31;
-  const T* Jb = J + (int64_t)b * kJP * nc;
   for (int e = threadIdx.x; e < n * ld; e += blockDim.x) A[e] = (T)0;
   __syncthreads();
-  for (int cell = threadIdx.x; cell < nc; cell += blockDim.x) {
+  for (int e = threadIdx.x; e < 5 * nc; e += blockDim.x) {
+    const int q = e / nc, cell = e - q * nc;
     const int j = cell / G.nx, i = cell - j * G.nx;
-    const int cs = cs_pos(i, j, G.nx, half);
-    const int nb[5] = {cell, i > 0 ? cell - 1 : -1, i < G.nx - 1 ? cell + 1 : -1,
-                       j > 0 ? cell - G.nx : -1, j < G.ny - 1 ? cell + G.nx : -1};
-    // the scaled system: identity diagonal blocks, At off the diagonal
-    A[(2 * cell) * ld + 2 * cell] = (T)1;
-    A[(2 * cell + 1) * ld + 2 * cell + 1] = (T)1;
-    for (int q = 1; q < 5; ++q) {
-      if (nb[q] < 0) continue;
-      for (int e = 0; e < 2; ++e)
-        for (int v = 0; v < 2; ++v)
-          A[(2 * cell + e) * ld + 2 * nb[q] + v] = Jb[(int64_t)(4 * q + 2 * e + v) * nc + cs];
+    if (q == 0) {   // the scaled system: identity diagonal blocks, At off the diagonal
+      A[(2 * cell) * ld + 2 * cell] = (T)1;
+      A[(2 * cell + 1) * ld + 2 * cell + 1] = (T)1;
+      continue;
     }
+    const bool has = q == 1 ? i > 0 : q == 2 ? i < G.nx - 1 : q == 3 ? j > 0 : j < G.ny - 1;
+    const int nb = cell + (q == 1 ? -1 : q == 2 ? 1 : q == 3 ? -G.nx : G.nx);
+    if (!has) continue;
+    const T* a = Jb + (int64_t)(4 * q) * nc + cs_pos(i, j, G.nx, half);
+    for (int m = 0; m < 4; ++m) A[(2 * cell + (m >> 1)) * ld + 2 * nb + (m & 1)] = a[(int64_t)m * nc];
   }
   __syncthreads();
+  const int step_r = blockDim.x / n, step_c = blockDim.x - step_r * n;
+  const int r0 = threadIdx.x / n, c0 = threadIdx.x - r0 * n;
   for (int k = 0; k < n; ++k) {
-    if (threadIdx.x < 32) {
-      // pivot: largest |A[r][k]|, r >= k, lowest index on ties
-      T bv = (T)-1;
-      int br = k;
-      for (int r = k + l; r < n; r += 32) {
-        const T v = fabs(A[r * ld + k]);
-        if (v > bv) { bv = v; br = r; }
-      }
+    // pivot: largest |A[r][k]|, r >= k, lowest index on ties
+    T bv = (T)-1;
+    int br = k;
+    for (int r = k + l; r < n; r += 32) {
+      const T v = fabs(A[r * ld + k]);
+      if (v > bv) { bv = v; br = r; }
+    }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const T ov = __shfl_down_sync(0xffffffffu, bv, o);
-        const int orr = __shfl_down_sync(0xffffffffu, br, o);
-        if (ov > bv || (ov == bv && orr < br)) { bv = ov; br = orr; }
-      }
-      br = __shfl_sync(0xffffffffu, br, 0);
-      // column k of the rows after the swap of rows k and br
-      for (int r = l; r < n; r += 32) fcol[r] = r == k ? (T)0 : A[(r == br ? k : r) * ld + k];
-      if (l == 0) {
-        const T d = A[br * ld + k];
-        pv[k] = br;
-        rinv_sh[0] = d != (T)0 ? (T)1 / d : (T)0;
-      }
+    for (int o = 16; o > 0; o >>= 1) {
+      const T ov = __shfl_xor_sync(0xffffffffu, bv, o);
+      const int orr = __shfl_xor_sync(0xffffffffu, br, o);
+      if (ov > bv || (ov == bv && orr < br)) { bv = ov; br = orr; }
     }
-    __syncthreads();
-    const int br = pv[k];
-    const T rinv = rinv_sh[0];
-    for (int col = threadIdx.x; col < n; col += blockDim.x) {
-      // swap rows k and br; the new pivot row divided by the pivot, its own
-      // column becoming 1 / pivot
-      const T a = A[br * ld + col];
-      if (br != k) A[br * ld + col] = A[k * ld + col];
-      A[k * ld + col] = (col == k ? (T)1 : a) * rinv;
+    const T d = A[br * ld + k];
+    const T rinv = d != (T)0 ? (T)1 / d : (T)0;
+    if (threadIdx.x == 0) pv[k] = br;
+    int r = r0, c = c0;
+    while (r < n) {
+      const int src = r == br ? k : r;
+      const T prow = (c == k ? (T)1 : A[br * ld + c]) * rinv;
+      const T v = c == k ? (T)0 : A[src * ld + c];
+      Y[r * ld + c] = r == k ? prow : fma(-A[src * ld + k], prow, v);
+      r += step_r;
+      c += step_c;
+      if (c >= n) { c -= n; ++r; }
     }
-    __syncthreads();
-    // every other row: subtract f times the pivot row, its column k
-    // becoming -f / pivot
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-      const int row = e / n, col = e - row * n;
-      if (row == k) continue;
-      const T v = col == k ? (T)0 : A[row * ld + col];
-      A[row * ld + col] = fma(-fcol[row], A[k * ld + col], v);
-    }
+    T* s = A;
+    A = Y;
+    Y = s;
     __syncthreads();
   }
   // column c of the inverse is column q(c) of the eliminated matrix, with
@@ -518,11 +528,90 @@ k_coarse_inv(unsigned long long* ctr, Geom G, int B, const int* __restrict__ act
     qcol[c] = x;
   }
   __syncthreads();
-  T* out = AinvT + (int64_t)b * kMaxCoarseUnknowns * kMaxCoarseUnknowns;
   for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
     const int v = e / n, u = e - v * n;
     out[e] = A[u * ld + qcol[v]];
   }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kInvThreads)
+k_coarse_inv(unsigned long long* ctr, Geom G, int B, const int* __restrict__ active,
+             const T* __restrict__ J, T* __restrict__ AinvT, const int* __restrict__ refresh) {
+  HENRY_COUNT_LAUNCH(ctr);
+  extern __shared__ __align__(16) unsigned char inv_sh[];
+  const int b = blockIdx.x;
+  if (!active[b] || (refresh && !refresh[b])) return;
+  coarse_inverse<T>(G, J + (int64_t)b * kJP * G.ncell(),
+                    AinvT + (int64_t)b * kMaxCoarseUnknowns * kMaxCoarseUnknowns, inv_sh);
+}
+
+// Jacobian of one cell of a coarse multigrid level from its own state and
+// fields, row-scaled into the sample's operators Jb.
+template <typename T>
+struct CoarseOps {
+  CoarseStates st;
+  const double *phi[kMaxLevels], *K[kMaxLevels], *tx[kMaxLevels], *dx[kMaxLevels], *ty[kMaxLevels],
+      *dy[kMaxLevels];
+  T* J[kMaxLevels];
+  double vtau[kMaxLevels];           // cell volume / time step
+  int first[kMaxLevels];             // first block of the level
+};
+
+template <typename T>
+__device__ __forceinline__ void coarse_jac_cell(const Phys& P, const CoarseOps<T>& M, int k, int b,
+                                                int cell) {
+  const Geom G = M.st.g[k];
+  const int ncell = G.ncell();
+  const int j = cell / G.nx, i = cell - j * G.nx;
+  const int64_t o = (int64_t)b * ncell;
+  const double *c = M.st.c[k], *qx = M.st.qx[k], *qy = M.st.qy[k];
+  CellIn in;
+  gather_cell(G, i, j, c + o, c + o, M.phi[k] + o, M.K[k] + o, M.tx[k] + o, M.dx[k] + o, M.ty[k] + o,
+              M.dy[k] + o, in);   // (the fluxes are given: no pressures)
+  in.c_old = in.c;
+  in.qin = 0.0;
+  in.qE = qx[o + cell];
+  in.qN = in.hasN ? qy[o + cell] : 0.0;
+  in.qW = in.hasW ? qx[o + cell - 1] : 0.0;
+  in.qS = in.hasS ? qy[o + cell - G.nx] : 0.0;
+  double Rp, Rc;
+  T Jc[20];
+  cell_residual<T, true, true>(P, G, M.vtau[k], in, Rp, Rc, Jc);
+  T* Jb = M.J[k] + (int64_t)b * kJP * ncell + cs_pos(i, j, G.nx, G.half());
+  T d[4];
+  store_operator<T>(Jb, ncell, Jc, d);
+}
+
+// Operators of levels 0..nl-2, and with AinvT the inverse of level 0: block b
+// < B the coarsest level of sample b (and its inverse, whose chain of n
+// dependent pivots then runs beside the other levels' cells), the blocks from
+// first[k] on level k. Dynamic shared memory coarse_inv_smem_bytes<T>(n).
+template <typename T>
+__global__ void __launch_bounds__(kInvThreads)
+k_coarse_ops(unsigned long long* ctr, Phys P, const __grid_constant__ CoarseOps<T> M, int B,
+             const int* __restrict__ active, T* __restrict__ AinvT, const int* __restrict__ refresh) {
+  HENRY_COUNT_LAUNCH(ctr);
+  extern __shared__ __align__(16) unsigned char inv_sh[];
+  if ((int)blockIdx.x < B) {
+    const int b = blockIdx.x;
+    if (!active[b] || (refresh && !refresh[b])) return;
+    for (int cell = threadIdx.x; cell < M.st.g[0].ncell(); cell += blockDim.x)
+      coarse_jac_cell<T>(P, M, 0, b, cell);
+    if (!AinvT) return;
+    __syncthreads();   // the block's own operators
+    coarse_inverse<T>(M.st.g[0], M.J[0] + (int64_t)b * kJP * M.st.g[0].ncell(),
+                      AinvT + (int64_t)b * kMaxCoarseUnknowns * kMaxCoarseUnknowns, inv_sh);
+    return;
+  }
+  int k = 1;
+  while (k < M.st.nl - 2 && (int)blockIdx.x >= M.first[k + 1]) ++k;
+  const int64_t idx = (int64_t)((int)blockIdx.x - M.first[k]) * blockDim.x + threadIdx.x;
+  const int ncell = M.st.g[k].ncell();
+  if (idx >= (int64_t)B * ncell) return;
+  const int b = (int)(idx / ncell);
+  if (!active[b] || (refresh && !refresh[b])) return;
+  coarse_jac_cell<T>(P, M, k, b, (int)(idx - (int64_t)b * ncell));
 }
 
 // ---------------------------------------------------------------------------
@@ -848,7 +937,6 @@ k_prolong(unsigned long long* ctr, Geom Gc, Geom Gf, int B, const int* __restric
 // memory hold their mbarrier.
 // ---------------------------------------------------------------------------
 constexpr int kSmallCells = 512;   // largest level the shared-memory kernel accepts
-constexpr int kMaxLevels = 12;
 
 template <typename T>
 struct SmallMG {

@@ -170,6 +170,13 @@ static cudaError_t raise_smem_limit(const void* fn, size_t smem) {
 }
 
 int Solver::ensure(int B, cudaStream_t s) {
+  {
+    const bool f32 = tsize_ == sizeof(float);
+    const int n = 2 * geoms_[0].ncell();
+    const size_t smem = f32 ? coarse_inv_smem_bytes<float>(n) : coarse_inv_smem_bytes<double>(n);
+    CK(raise_smem_limit(f32 ? (const void*)k_coarse_ops<float> : (const void*)k_coarse_ops<double>, smem));
+    CK(raise_smem_limit(f32 ? (const void*)k_coarse_inv<float> : (const void*)k_coarse_inv<double>, smem));
+  }
   if (ks_ > 0) {
     SmallMG<float> Mf;
     SmallMG<double> Md;
@@ -468,28 +475,49 @@ void Solver::enqueue_vcycle(int k, int B, cudaStream_t s) {
 }
 
 // Coarse multigrid operators at the current iterate (linearised about the
-// restricted face fluxes).
+// restricted face fluxes); with_inv: and the coarsest level's inverse.
 template <typename T>
-void Solver::enqueue_coarse_ops(int B, cudaStream_t s, const int* refresh) {
+void Solver::enqueue_coarse_ops(int B, cudaStream_t s, const int* refresh, bool with_inv) {
   const int nl = (int)levels_.size();
-  for (int k = nl - 1; k >= 1; --k) {
-    MGLevel& F = levels_[k];
-    MGLevel& C = levels_[k - 1];
-    k_restrict_state<<<grid1((int64_t)B * C.g.ncell()), kBlock, 0, s>>>(
-        counter_, F.g, C.g, B, active_, F.c, F.qx, F.qy, C.c, C.qx, C.qy, refresh);
-    k_jac<T><<<grid1((int64_t)B * C.g.ncell()), kBlock, 0, s>>>(
-        counter_, phys_, C.g, C.g.hx * C.g.hy / tau_, B, active_, C.p, C.c, C.phi, C.K, C.tx, C.dx, C.ty, C.dy,
-        C.qx, C.qy, (T*)C.J, refresh);
+  if (nl == 1) {   // the finest level is the coarsest
+    if (with_inv) enqueue_coarse_inv<T>(B, s, refresh);
+    return;
   }
+  CoarseOps<T> M = {};
+  M.st.nl = nl;
+  int blocks = B;
+  for (int k = 0; k < nl; ++k) {
+    const MGLevel& L = levels_[k];
+    M.st.g[k] = L.g;
+    M.st.c[k] = L.c;
+    M.st.qx[k] = L.qx;
+    M.st.qy[k] = L.qy;
+    M.phi[k] = L.phi;
+    M.K[k] = L.K;
+    M.tx[k] = L.tx;
+    M.dx[k] = L.dx;
+    M.ty[k] = L.ty;
+    M.dy[k] = L.dy;
+    M.J[k] = (T*)L.J;
+    M.vtau[k] = L.g.hx * L.g.hy / tau_;
+    M.first[k] = blocks;
+    if (k > 0 && k < nl - 1) blocks += (int)(((int64_t)B * L.g.ncell() + kInvThreads - 1) / kInvThreads);
+  }
+  for (int top = nl - 1; top >= 1;) {
+    const int depth = top < kRestrictDepth ? top : kRestrictDepth;
+    const int64_t cells = (int64_t)B * levels_[top - 1].g.ncell();
+    k_restrict_states<<<grid1(cells), kBlock, 0, s>>>(counter_, M.st, top, depth, B, active_, refresh);
+    top -= depth;
+  }
+  k_coarse_ops<T><<<blocks, kInvThreads, coarse_inv_smem_bytes<T>(2 * levels_[0].g.ncell()), s>>>(
+      counter_, phys_, M, B, active_, with_inv ? (T*)cinv_ : nullptr, refresh);
 }
 
 template <typename T>
 void Solver::enqueue_coarse_inv(int B, cudaStream_t s, const int* refresh) {
-  {
-    const int n = 2 * levels_[0].g.ncell();
-    k_coarse_inv<T><<<B, kBlock, coarse_inv_smem_bytes<T>(n), s>>>(
-        counter_, levels_[0].g, B, active_, (const T*)levels_[0].J, (T*)cinv_, refresh);
-  }
+  const int n = 2 * levels_[0].g.ncell();
+  k_coarse_inv<T><<<B, kInvThreads, coarse_inv_smem_bytes<T>(n), s>>>(
+      counter_, levels_[0].g, B, active_, (const T*)levels_[0].J, (T*)cinv_, refresh);
 }
 
 template <typename T>
@@ -568,8 +596,7 @@ void Solver::enqueue_rebuild(int B, cudaStream_t s) {
   if (refresh) {
     launch_resjac<T>(B, refresh, nullptr, s);
   }
-  enqueue_coarse_ops<T>(B, s, refresh);
-  enqueue_coarse_inv<T>(B, s, refresh);
+  enqueue_coarse_ops<T>(B, s, refresh, true);
 }
 
 // Linear solve of the defect correction (V-cycles or BiCGStab) and the
@@ -1195,7 +1222,7 @@ int Solver::adjoint_t(const double* xi, const double* logk, int B, int qoi, int 
       launch_resjac<T>(B, nullptr, nullptr, s);
       k_residual<double, 2, true, true, false, true><<<dim3(tile_j_.warps(), B), 32, 0, s>>>(
           counter_, phys_, G, G.hx * G.hy / tau_, tile_j_, res_args(), J64_, res_, nullptr);
-      enqueue_coarse_ops<T>(B, s, nullptr);
+      enqueue_coarse_ops<T>(B, s, nullptr, false);
       for (size_t k = 0; k < levels_.size(); ++k)
         k_transpose<T><<<grid1((int64_t)B * levels_[k].g.ncell()), kBlock, 0, s>>>(
             counter_, levels_[k].g, B, active_, (const T*)levels_[k].J, (T*)JT_[k]);

@@ -110,7 +110,7 @@ class Solver {
                                   int status_or, cudaStream_t s);
   template <typename T> int setup_t(const double* xi, const double* logk, int B, cudaStream_t s);
   template <typename T> int step_t(int B, cudaStream_t s);
-  template <typename T> void enqueue_coarse_ops(int B, cudaStream_t s, const int* refresh);
+  template <typename T> void enqueue_coarse_ops(int B, cudaStream_t s, const int* refresh, bool with_inv);
   template <typename T> void enqueue_coarse_inv(int B, cudaStream_t s, const int* refresh);
   template <typename T> void enqueue_vcycles(int B, cudaStream_t s);
   template <typename T> void enqueue_precond(int B, cudaStream_t s);
