@@ -165,13 +165,31 @@ static __global__ void k_init_state(unsigned long long* ctr, Phys P, Geom G, int
 // ---------------------------------------------------------------------------
 // per time step
 // ---------------------------------------------------------------------------
-// Start of an implicit Euler step: c_old = c^{n-1} (with mo / so given, also
-// the old-time storage terms of k_residual). With `extrapolate`, from
-// the third step on (both u^{n-1} and u^{n-2} are solutions; the first
-// step's pressure guess is not) the Newton initial guess is extrapolated
-// linearly in time, u = 2 u^{n-1} - u^{n-2}, with c clamped to [0, 1]
-// (p_prev keeps p^{n-2}, c_old c^{n-2} on entry). `step` counts completed
-// steps (k_end_step increments it).
+// Start of an implicit Euler step: c_old = c^n and, with mo / so given, the
+// old time level's storage terms of k_residual (vt_out, V phi / tau, changes
+// with the fields only: written in a solve's first step). From the third step
+// on Newton's initial guess is extrapolated in time (p_prev keeps p^(n-1) on
+// entry, c_old c^(n-1)). `step` counts completed steps (k_end_step increments
+// it). Bound by HBM on large grids: the weights of the extrapolation come with
+// the launch (four FP64 divisions per cell made it FP64-bound: 1024x512 cells
+// x 16, 607 us; 266 us so, of which about 230 are its 23 arrays).
+struct GuessWeights {
+  double w[kMaxGuessHist + 2][kMaxGuessHist + 2];   // [q][k] = (-1)^k C(q+1, k+1)
+};
+
+__host__ inline GuessWeights guess_weights() {
+  GuessWeights g = {};
+  for (int q = 1; q < kMaxGuessHist + 2; ++q) {
+    double w = q + 1.0;
+    g.w[q][0] = w;
+    for (int k = 1; k <= q; ++k) {
+      w = -w * (q + 1 - k) / (k + 1);
+      g.w[q][k] = w;
+    }
+  }
+  return g;
+}
+
 template <int D = 0>   // history arrays in use (hx.depth)
 static __global__ void k_begin_step(unsigned long long* ctr, Geom G, int B, double* __restrict__ p,
                              double* __restrict__ c, double* __restrict__ p_prev,
@@ -182,7 +200,8 @@ static __global__ void k_begin_step(unsigned long long* ctr, Geom G, int B, doub
                              double tau, const double* __restrict__ phi = nullptr,
                              double vtau = 0.0, double rho0 = 0.0, double drho = 0.0,
                              double* __restrict__ mo = nullptr, double* __restrict__ so = nullptr,
-                             double* __restrict__ vt_out = nullptr, GuessHist hx = {}) {
+                             double* __restrict__ vt_out = nullptr, GuessHist hx = {},
+                             const __grid_constant__ GuessWeights gw = {}) {
   HENRY_COUNT_LAUNCH(ctr);
   const int64_t n = (int64_t)B * G.ncell();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -214,12 +233,11 @@ static __global__ void k_begin_step(unsigned long long* ctr, Geom G, int B, doub
   if (q > *step - 1) q = *step - 1;
   if (q > 1 + D) q = 1 + D;
   if (q >= 1) {
-    double w = q + 1.0;                 // C(q+1, 1)
-    double ec = w * cn, ep = w * pn;
+    double ec = gw.w[q][0] * cn, ep = gw.w[q][0] * pn;
 #pragma unroll
     for (int k = 1; k <= 1 + D; ++k) {
       if (k > q) break;
-      w = -w * (q + 1 - k) / (k + 1);   // (-1)^k C(q+1, k+1)
+      const double w = gw.w[q][k];
       ec += w * hc[k - 1];
       ep += w * hp[k - 1];
     }
@@ -240,7 +258,7 @@ static __global__ void k_begin_step(unsigned long long* ctr, Geom G, int B, doub
     const double m = vt * (rho0 + drho * cn);
     mo[idx] = m;
     so[idx] = m * cn;
-    vt_out[idx] = vt;
+    if (*step == 0) vt_out[idx] = vt;
   }
   const int b = (int)(idx / G.ncell());
   if (idx - (int64_t)b * G.ncell() == 0) {
@@ -1052,7 +1070,7 @@ __global__ void k_update(unsigned long long* ctr, Geom G, int B, const int* __re
 }
 
 // ---------------------------------------------------------------------------
-// quantities of interest (section 4): one block per sample
+// quantities of interest (section 4)
 // ---------------------------------------------------------------------------
 constexpr double kFreshC = 0.012178;   // fresh-water threshold of Eq. integral_fw
 constexpr double kBoxHalf = 0.1;        // half-width of the boxes of Eq. integral_box
@@ -1068,16 +1086,25 @@ __device__ __forceinline__ double bilinear(const Geom& G, const double* c, doubl
          tx * ty * c[id + G.nx + 1];
 }
 
+constexpr int kQoiCells = 2048;   // cells per block of k_qoi
+constexpr int kQoiSums = 19;      // Q_S, mass, toe, fresh cells, 15 boxes
+
+// Partial sums of the QoI integrals, one block per kQoiCells cells of a
+// sample: part [B][chunks][kQoiSums]; and the output fields. FP64-bound: the
+// box overlaps are formed only for cells that reach a box (x >= 0.8, y <=
+// 0.6), fresh cells are counted in integers. (One block per sample took 6.03
+// ms on 1024x512 cells x 16, this form 0.60.)
 static __global__ void __launch_bounds__(kBlock)
-k_qoi(unsigned long long* ctr, Phys P, Geom G, int B, const double* __restrict__ p,
-      const double* __restrict__ c, const double* __restrict__ phi, double* __restrict__ q,
-      double* __restrict__ c_out, double* __restrict__ p_out, int qstride) {
+k_qoi(unsigned long long* ctr, Phys P, Geom G, const double* __restrict__ p,
+      const double* __restrict__ c, const double* __restrict__ phi, double* __restrict__ part,
+      double* __restrict__ c_out, double* __restrict__ p_out) {
   HENRY_COUNT_LAUNCH(ctr);
-  __shared__ double sh[kBlock / 32];
-  const int b = blockIdx.x;
+  __shared__ double sh[kBlock / 32][kQoiSums];
+  const int b = blockIdx.y;
   const int ncell = G.ncell();
   const int64_t o = (int64_t)b * ncell;
-  double s0 = 0, s1 = 0, s2 = 0, fw = 0;
+  double s0 = 0, s1 = 0, s2 = 0;
+  int fw = 0;
   double box[15];
 #pragma unroll
   for (int m = 0; m < 15; ++m) box[m] = 0.0;
@@ -1085,47 +1112,73 @@ k_qoi(unsigned long long* ctr, Phys P, Geom G, int B, const double* __restrict__
   // 12points (frame y in [0, 1]), half-width 0.1, clipped to the domain
   const double bx[5] = {0.90, 1.15, 1.40, 1.65, 1.90};
   const double by[3] = {0.05, 0.25, 0.50};
-  for (int cell = threadIdx.x; cell < ncell; cell += blockDim.x) {
+  const int c0 = blockIdx.x * kQoiCells, c1 = c0 + kQoiCells < ncell ? c0 + kQoiCells : ncell;
+  // first column and last row that can reach a box (whole cells of slack)
+  const int ibox = (int)((bx[0] - kBoxHalf) / G.hx) - 1, jbox = (int)((by[2] + kBoxHalf) / G.hy) + 1;
+  for (int cell = c0 + threadIdx.x; cell < c1; cell += blockDim.x) {
     const double cv = c[o + cell];
-    const double rho = P.rho0 + P.drho * cv;
     const int j = cell / G.nx, i = cell - j * G.nx;
-    const double x = (i + 0.5) * G.hx;
-    s0 += cv * rho;
-    s1 += phi[o + cell] * rho * cv;
-    s2 += cv * (P.Lx - x);
-    fw += cv <= kFreshC ? 1.0 : 0.0;
-    const double xl = i * G.hx, yl = j * G.hy;
+    const double w = cv * (P.rho0 + P.drho * cv);
+    s0 += w;
+    s1 += phi[o + cell] * w;
+    s2 += cv * (P.Lx - (i + 0.5) * G.hx);
+    fw += cv <= kFreshC ? 1 : 0;
+    if (i >= ibox && j <= jbox) {
+      const double xl = i * G.hx, yl = j * G.hy;
 #pragma unroll
-    for (int r = 0; r < 3; ++r) {
-      const double oy = fmax(fmin(yl + G.hy, by[r] + kBoxHalf) - fmax(yl, by[r] - kBoxHalf), 0.0);
-      if (oy == 0.0) continue;
+      for (int r = 0; r < 3; ++r) {
+        const double oy = fmin(yl + G.hy, by[r] + kBoxHalf) - fmax(yl, by[r] - kBoxHalf);
+        if (oy <= 0.0) continue;
 #pragma unroll
-      for (int k = 0; k < 5; ++k) {
-        const double ox = fmax(fmin(xl + G.hx, bx[k] + kBoxHalf) - fmax(xl, bx[k] - kBoxHalf), 0.0);
-        box[5 * r + k] += cv * rho * oy * ox;
+        for (int k = 0; k < 5; ++k) {
+          const double ox = fmin(xl + G.hx, bx[k] + kBoxHalf) - fmax(xl, bx[k] - kBoxHalf);
+          if (ox > 0.0) box[5 * r + k] += w * oy * ox;
+        }
       }
     }
     if (c_out) c_out[o + cell] = cv;
     if (p_out) p_out[o + cell] = p[o + cell] + P.rho0 * P.g * (P.Ly - (j + 0.5) * G.hy);
   }
+  const int wp = threadIdx.x >> 5, l = threadIdx.x & 31;
+  auto reduce = [&](int m, double v) {
+#pragma unroll
+    for (int t = 16; t > 0; t >>= 1) v += __shfl_down_sync(0xffffffffu, v, t);
+    if (l == 0) sh[wp][m] = v;
+  };
+  reduce(0, s0);
+  reduce(1, s1);
+  reduce(2, s2);
+  reduce(3, (double)__reduce_add_sync(0xffffffffu, fw) * (l == 0 ? 1.0 : 0.0));
+#pragma unroll
+  for (int m = 0; m < 15; ++m) {
+    if (__any_sync(0xffffffffu, box[m] != 0.0)) reduce(4 + m, box[m]);
+    else if (l == 0) sh[wp][4 + m] = 0.0;
+  }
+  __syncthreads();
+  if (threadIdx.x < kQoiSums) {
+    double v = 0.0;
+    for (int u = 0; u < kBlock / 32; ++u) v += sh[u][threadIdx.x];
+    part[((int64_t)b * gridDim.x + blockIdx.x) * kQoiSums + threadIdx.x] = v;
+  }
+}
+
+// The QoIs of a sample (a block of one warp per sum) from its partial sums.
+static __global__ void __launch_bounds__(32 * kQoiSums)
+k_qoi_sum(unsigned long long* ctr, Geom G, int chunks, const double* __restrict__ part,
+          const double* __restrict__ c, double* __restrict__ q, int qstride) {
+  HENRY_COUNT_LAUNCH(ctr);
+  const int b = blockIdx.x, m = threadIdx.x >> 5, l = threadIdx.x & 31;
+  const double* pb = part + (int64_t)b * chunks * kQoiSums + m;
+  double v = 0.0;
+  for (int k = l; k < chunks; k += 32) v += pb[(int64_t)k * kQoiSums];
+#pragma unroll
+  for (int t = 16; t > 0; t >>= 1) v += __shfl_down_sync(0xffffffffu, v, t);
+  double* qb = q + (int64_t)b * qstride;     // [B][...][kNQ]: sample stride qstride
   const double V = G.hx * G.hy;
-  s0 = block_sum(s0, sh);
-  s1 = block_sum(s1, sh);
-  s2 = block_sum(s2, sh);
-  fw = block_sum(fw, sh);
-#pragma unroll
-  for (int m = 0; m < 15; ++m) box[m] = block_sum(box[m], sh);
-  if (threadIdx.x == 0) {
-    double* qb = q + (int64_t)b * qstride;   // [B][...][kNQ]: sample stride qstride
-    qb[0] = s0 * V;
-    qb[1] = s1 * V;
-    qb[2] = s2 * V;
-    qb[3] = bilinear(G, c + o, 1.40, 0.05);
-    qb[4] = bilinear(G, c + o, 1.65, 0.25);
-    qb[5] = bilinear(G, c + o, 1.90, 0.50);
-    qb[6] = fw * V;
-#pragma unroll
-    for (int m = 0; m < 15; ++m) qb[7 + m] = box[m];
+  if (l == 0) qb[m < 3 ? m : m == 3 ? 6 : m + 3] = m < 4 ? v * V : v;
+  if (m < 3 && l == 1) {
+    const double x[3] = {1.40, 1.65, 1.90}, y[3] = {0.05, 0.25, 0.50};
+    qb[3 + m] = bilinear(G, c + (int64_t)b * G.ncell(), x[m], y[m]);
   }
 }
 

@@ -268,6 +268,7 @@ int Solver::ensure(int B, cudaStream_t s) {
   const size_t o_qin = take((size_t)F.ny * Bz * 8);
   const size_t o_qin0 = take((size_t)F.ny * Bz * 8);
   const size_t o_part = take((size_t)nchunk_ * Bz * 8);
+  const size_t o_qoi = take((size_t)qoi_chunks() * kQoiSums * Bz * 8);
   const size_t o_res0 = take(Bz * 8);
   const size_t o_resl = take(Bz * 8);
   const size_t o_cinv = take(Bz * kMaxCoarseUnknowns * kMaxCoarseUnknowns * 8);
@@ -327,6 +328,7 @@ int Solver::ensure(int B, cudaStream_t s) {
   qin_ = (double*)(a + o_qin);
   qin0_ = (double*)(a + o_qin0);
   partial_ = (double*)(a + o_part);
+  qoi_part_ = (double*)(a + o_qoi);
   res0_ = (double*)(a + o_res0);
   res_last_ = (double*)(a + o_resl);
   cinv_ = a + o_cinv;
@@ -890,6 +892,19 @@ int Solver::setup_t(const double* xi, const double* logk, int B, cudaStream_t s)
   return HENRY_OK;
 }
 
+// QoIs (and fields) of the current state; qstride: doubles from one sample's
+// QoIs to the next's.
+void Solver::launch_qoi(int B, double* q, double* c_out, double* p_out, int qstride, cudaStream_t s) {
+  const MGLevel& F = levels_.back();
+  const int chunks = qoi_chunks();
+  k_qoi<<<dim3(chunks, B), kBlock, 0, s>>>(counter_, phys_, F.g, F.p, F.c, F.phi, qoi_part_, c_out, p_out);
+  k_qoi_sum<<<B, 32 * kQoiSums, 0, s>>>(counter_, F.g, chunks, qoi_part_, F.c, q, qstride);
+}
+
+int Solver::qoi_chunks() const {
+  return (levels_.back().g.ncell() + kQoiCells - 1) / kQoiCells;
+}
+
 // Begin every sample's step (k_begin_step, instantiated for the depth of
 // the Newton guess's history).
 void Solver::launch_begin_step(int B, cudaStream_t s) {
@@ -899,7 +914,7 @@ void Solver::launch_begin_step(int B, cudaStream_t s) {
     kern<<<grid1((int64_t)B * G.ncell()), kBlock, 0, s>>>(
         counter_, G, B, F.p, F.c, p_prev_, c_old_, status_w_, active_, it_step_, step_,
         cfg_.guess_extrapolation, cfg_.field_model == 1 ? qin0_ : nullptr, qin_, tau_, F.phi,
-        G.hx * G.hy / tau_, phys_.rho0, phys_.drho, mo_, so_, vt_, hx_);
+        G.hx * G.hy / tau_, phys_.rho0, phys_.drho, mo_, so_, vt_, hx_, guess_weights());
   };
   switch (hx_.depth) {
     case 0: go(k_begin_step<0>); break;
@@ -941,10 +956,8 @@ int Solver::run_t(const double* xi, const double* logk, int B, double* q, double
     rc = step_t<T>(B, s);
     if (rc) return rc;
     if (series_ && (n + 1) % series_every_ == 0) {
-      MGLevel& F = levels_.back();
       const int k = (n + 1) / series_every_ - 1;
-      k_qoi<<<B, kBlock, 0, s>>>(counter_, phys_, F.g, B, F.p, F.c, F.phi, series_ + k * kNQ,
-                                 nullptr, nullptr, nout * kNQ);
+      launch_qoi(B, series_ + k * kNQ, nullptr, nullptr, nout * kNQ, s);
     }
   }
   return finish(B, q, c_out, p_out, status, iters, status_or, s);
@@ -960,9 +973,7 @@ int Solver::begin(const double* xi, const double* logk, int B, cudaStream_t s) {
 
 int Solver::finish(int B, double* q, double* c_out, double* p_out, int* status, int* iters,
                    int status_or, cudaStream_t s) {
-  MGLevel& F = levels_.back();
-  const Geom& G = F.g;
-  k_qoi<<<B, kBlock, 0, s>>>(counter_, phys_, G, B, F.p, F.c, F.phi, q, c_out, p_out, kNQ);
+  launch_qoi(B, q, c_out, p_out, kNQ, s);
   k_copy_int<<<grid1(B), kBlock, 0, s>>>(counter_, B, status_w_, status, status_or);
   if (iters) k_copy_int<<<grid1(B), kBlock, 0, s>>>(counter_, B, iters_w_, iters, 0);
   CK(cudaGetLastError());
@@ -1182,7 +1193,7 @@ int Solver::adjoint_t(const double* xi, const double* logk, int B, int qoi, int 
     if (st % kc == 0) { if ((rc = save(ck(st / kc), true))) return rc; }
     else if (st == nt_) { if ((rc = save(ck(nck - 1), true))) return rc; }
   }
-  k_qoi<<<B, kBlock, 0, s>>>(counter_, phys_, G, B, F.p, F.c, F.phi, qtmp_, nullptr, nullptr, kNQ);
+  launch_qoi(B, qtmp_, nullptr, nullptr, kNQ, s);
   CK(cudaMemcpy2DAsync(q, sizeof(double), qtmp_ + qoi, kNQ * sizeof(double), sizeof(double), B,
                        cudaMemcpyDeviceToDevice, s));
   // seed and zero the sensitivities

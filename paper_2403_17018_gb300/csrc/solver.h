@@ -156,6 +156,8 @@ class Solver {
   GuessHist hx_ = {};           // u^(n-2), ... for guesses of order >= 2
   // previous states the Newton guess reads beyond u^(n-1)
   void launch_begin_step(int B, cudaStream_t s);
+  void launch_qoi(int B, double* q, double* c_out, double* p_out, int qstride, cudaStream_t s);
+  int qoi_chunks() const;
   int guess_depth() const {
     const int d = cfg_.guess_extrapolation - 1;
     return d < 0 ? 0 : (d > kMaxGuessHist ? kMaxGuessHist : d);
@@ -172,6 +174,7 @@ class Solver {
   double* qin_ = nullptr;
   double* qin0_ = nullptr;     // inflow base of the paper field model (time factor per step)
   double* partial_ = nullptr;
+  double* qoi_part_ = nullptr;  // partial sums of the QoI integrals
   double* res0_ = nullptr;
   double* res_last_ = nullptr;
   char* cinv_ = nullptr;      // transposed inverse of the coarsest operator (multigrid type)

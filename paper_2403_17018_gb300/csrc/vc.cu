@@ -535,7 +535,8 @@ int VcSolver::run(const double* xi, int B, double* q, double* c_out, double* p_o
   for (int stp = 0; stp < nt_; ++stp) {
     k_begin_step<<<gn, kBlock, 0, s>>>(counter_, G_, B, p_, c_, p_prev_, c_old_, status_w_,
                                        active_, it_step_, step_, cfg_.guess_extrapolation,
-                                       paper ? qin0_ : nullptr, qin_, tau_);
+                                       paper ? qin0_ : nullptr, qin_, tau_, nullptr, 0.0, 0.0, 0.0,
+                                       nullptr, nullptr, nullptr, GuessHist{}, guess_weights());
     for (;;) {
       k_vc_resjac<false, true><<<gr, kBlock, 0, s>>>(counter_, phys_, G_, tau_, B, vphi_, vol_,
                                                      tx_, dx_, ty_, dy_, qin_, p_, c_, c_old_,
