@@ -188,6 +188,7 @@ struct ResArgs {
   double* partial;        // [B][warps] sums of R_p^2 + R_c^2, or null
   double* qx;             // face fluxes (WANT_J of the multigrid layout), or null
   double* qy;
+  int guess;              // the guess xvec: 0, or with b on the red cells (its first half-sweep)
 };
 
 }  // namespace henry

@@ -725,8 +725,8 @@ __device__ __forceinline__ void resid_point(int i, int j, int nx, int ny, int nc
     rc -= Jc[(19 - P0) * ncell] * vc;
   }
   const T sp = rp, sc = rc;
-  rp = Jc[(20 - P0) * ncell] * sp + Jc[(21 - P0) * ncell] * sc;
-  rc = Jc[(22 - P0) * ncell] * sp + Jc[(23 - P0) * ncell] * sc;
+  rp = fma(Jc[(20 - P0) * ncell], sp, Jc[(21 - P0) * ncell] * sc);
+  rc = fma(Jc[(22 - P0) * ncell], sp, Jc[(23 - P0) * ncell] * sc);
 }
 
 // Reader of a sample's unknowns in the colour-split layout.
@@ -803,8 +803,8 @@ __device__ __forceinline__ void restrict_cell(const Geom& Gf, const Geom& Gc, in
   }
   const int csc = cs_pos(I, J, Gc.nx, Gc.half());
   const T* d = Jc + csc;
-  bc[csc] = d[0] * sp + d[ncc] * sc;
-  bc[ncc + csc] = d[2 * ncc] * sp + d[3 * ncc] * sc;
+  bc[csc] = fma(d[0], sp, d[ncc] * sc);
+  bc[ncc + csc] = fma(d[2 * ncc], sp, d[3 * ncc] * sc);
   xc[csc] = (T)0;
   xc[ncc + csc] = (T)0;
 }
@@ -829,8 +829,8 @@ __device__ __forceinline__ void prolong_value(const Geom& Gc, int i, int j,
   const int a0 = cs_pos(I, J, Gc.nx, hc), a1 = cs_pos(I2, J, Gc.nx, hc);
   const int a2 = cs_pos(I, J2, Gc.nx, hc), a3 = cs_pos(I2, J2, Gc.nx, hc);
   const T w0 = (T)0.5625, w1 = (T)0.1875, w3 = (T)0.0625;
-  vp = w0 * xc[a0] + w1 * (xc[a1] + xc[a2]) + w3 * xc[a3];
-  vc = w0 * xc[ncc + a0] + w1 * (xc[ncc + a1] + xc[ncc + a2]) + w3 * xc[ncc + a3];
+  vp = fma(w3, xc[a3], fma(w0, xc[a0], w1 * (xc[a1] + xc[a2])));
+  vc = fma(w3, xc[ncc + a3], fma(w0, xc[ncc + a0], w1 * (xc[ncc + a1] + xc[ncc + a2])));
 }
 
 // Fine cell `cell` of level k: x_f += P x_c, cell-centred bilinear
@@ -890,57 +890,140 @@ __global__ void k_coarse_solve(unsigned long long* ctr, Geom G, int B, const int
                        xvec + ob, ysh[w], l);
 }
 
+// The kernels below take a cell (or a pair) per thread of grid row
+// blockIdx.y, the sample, and split a position into row and column by a
+// multiplication (RowDiv): the 64-bit division of a flat index and the
+// divisions by the grid's width were most of a half-sweep's instructions.
+struct RowDiv {
+  int n;
+  unsigned magic;                     // ceil(2^32 / n): the estimate is the row or one too high
+  __host__ __device__ explicit RowDiv(int w)
+      : n(w), magic(w > 1 ? (unsigned)((0x100000000ull + w - 1) / w) : 0u) {}
+  __device__ __forceinline__ int row(int pos) const {
+    const int j = magic ? (int)__umulhi((unsigned)pos, magic) : pos;
+    return j - (j * n > pos);
+  }
+};
+
 // One red (colour 0) or black (colour 1) half-sweep of point-block
-// Gauss-Seidel on every sample.
+// Gauss-Seidel on every sample. Grid (half / kBlock, B). Bound by HBM on
+// large grids (FP32, 1024x512 x 16: 56 us for the 369 MB it moves) and by the
+// FP64 pipe in FP64 (256x128 x 16: 9.6 us, 16 instructions per update are 8.2).
 template <typename T>
 __global__ void __launch_bounds__(kBlock)
-k_smooth(unsigned long long* ctr, Geom G, int B, int colour, const int* __restrict__ active,
+k_smooth(unsigned long long* ctr, Geom G, RowDiv rd, int colour, const int* __restrict__ active,
          const T* __restrict__ J, const T* __restrict__ bvec, T* __restrict__ xvec) {
   HENRY_COUNT_LAUNCH(ctr);
-  const int half = G.half(), ncell = G.ncell();
-  const int64_t n = (int64_t)B * half;
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n) return;
-  const int b = (int)(idx / half);
-  if (!active[b]) return;
-  const int pos = (int)(idx - (int64_t)b * half);
+  const int half = G.half(), ncell = G.ncell(), hx2 = G.nx >> 1;
+  const int b = blockIdx.y, pos = blockIdx.x * blockDim.x + threadIdx.x;
+  if (pos >= half || !active[b]) return;
+  const int j = rd.row(pos), k = pos - j * hx2;
+  const int i = 2 * k + ((j + colour) & 1);
+  const int own = colour * half + pos;
   const int64_t ob = (int64_t)b * 2 * ncell;
-  smooth_cell<T>(G, colour, pos, J + (int64_t)b * kJP * ncell, bvec + ob, xvec + ob);
+  const T* bs = bvec + ob;
+  T* xs = xvec + ob;
+  const T* xo = xs + (1 - colour) * half;   // the other colour's half of each plane
+  T xp, xc;
+  gs_point<T>(i, j, G.nx, G.ny, ncell, J + (int64_t)b * kJP * ncell + own, bs[own], bs[ncell + own],
+              [&](int ii, int jj, T& vp, T& vc) {
+                const int q = jj * hx2 + (ii >> 1);
+                vp = xo[q];
+                vc = xo[ncell + q];
+              },
+              xp, xc);
+  xs[own] = xp;
+  xs[ncell + own] = xc;
 }
+
+// Residual of level Gf restricted to Gc (restrict_cell's operations), the
+// coarse right-hand side scaled and the coarse guess: zero, or with `guess`
+// zero after the first red half-sweep (x_red = b_red), which then need not
+// be run. FP32 takes a thread per coarse cell. FP64, which two children's
+// loads leave with half the warps, takes two: a red child each (red_only;
+// else two children each), whose residuals they exchange, and one variable
+// of the result each (512x256 x 16: 49 us against 54 with one thread, FP32
+// 109 against 93). rd: division by the coarse width. Grid
+// (threads / kBlock, B).
+template <typename T>
+constexpr int kRestrictThreads = sizeof(T) == sizeof(double) ? 2 : 1;
 
 template <typename T>
 __global__ void __launch_bounds__(kBlock)
-k_resid_restrict(unsigned long long* ctr, Geom Gf, Geom Gc, int B, const int* __restrict__ active,
+k_resid_restrict(unsigned long long* ctr, Geom Gf, Geom Gc, RowDiv rd, const int* __restrict__ active,
                  const T* __restrict__ Jf, const T* __restrict__ bf, const T* __restrict__ xf,
-                 const T* __restrict__ Jc, T* __restrict__ bc, T* __restrict__ xc, int red_only) {
+                 const T* __restrict__ Jc, T* __restrict__ bc, T* __restrict__ xc, int red_only,
+                 int guess) {
   HENRY_COUNT_LAUNCH(ctr);
+  constexpr bool kTwo = kRestrictThreads<T> == 2;
   const int ncc = Gc.ncell(), ncf = Gf.ncell();
-  const int64_t n = (int64_t)B * ncc;
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n) return;
-  const int b = (int)(idx / ncc);
-  if (!active[b]) return;
-  const int cell = (int)(idx - (int64_t)b * ncc);
-  restrict_cell<T>(Gf, Gc, cell, Jf + (int64_t)b * kJP * ncf, bf + (int64_t)b * 2 * ncf,
-                   xf + (int64_t)b * 2 * ncf, Jc + (int64_t)b * kJP * ncc, bc + (int64_t)b * 2 * ncc,
-                   xc + (int64_t)b * 2 * ncc, red_only != 0);
+  const int b = blockIdx.y, t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (!active[b]) return;                     // uniform over the block
+  const int own = kTwo ? t >> 1 : t, part = kTwo ? t & 1 : 0;
+  const int cell = own < ncc ? own : ncc - 1;
+  const int J = rd.row(cell), I = cell - J * Gc.nx;
+  const T* Js = Jf + (int64_t)b * kJP * ncf;
+  const T* bs = bf + (int64_t)b * 2 * ncf;
+  const T* xs = xf + (int64_t)b * 2 * ncf;
+  const unsigned all = 0xffffffffu;
+  T sp, sc;
+  if (kTwo) {
+    T rp, rc;                                 // child 0 (2I, 2J) or 3 (2I + 1, 2J + 1)
+    residual_cell<T>(Gf, 2 * I + part, 2 * J + part, Js, bs, xs, rp, rc);
+    const T op = __shfl_xor_sync(all, rp, 1), oc = __shfl_xor_sync(all, rc, 1);
+    if (red_only) {
+      sp = part ? op + rp : rp + op;
+      sc = part ? oc + rc : rc + oc;
+    } else {
+      T up, uc;                               // child 1 (2I + 1, 2J) or 2 (2I, 2J + 1)
+      residual_cell<T>(Gf, 2 * I + 1 - part, 2 * J + part, Js, bs, xs, up, uc);
+      const T vp = __shfl_xor_sync(all, up, 1), vc = __shfl_xor_sync(all, uc, 1);
+      sp = part ? ((op + vp) + up) + rp : ((rp + up) + vp) + op;
+      sc = part ? ((oc + vc) + uc) + rc : ((rc + uc) + vc) + oc;
+    }
+  } else {
+    sp = 0, sc = 0;
+#pragma unroll
+    for (int c4 = 0; c4 < 4; ++c4) {
+      if (red_only && (c4 == 1 || c4 == 2)) continue;
+      T rp, rc;
+      residual_cell<T>(Gf, 2 * I + (c4 & 1), 2 * J + (c4 >> 1), Js, bs, xs, rp, rc);
+      sp += rp;
+      sc += rc;
+    }
+  }
+  if (own >= ncc) return;
+  const int csc = cs_pos(I, J, Gc.nx, Gc.half());
+  const bool red = guess && ((I + J) & 1) == 0;
+  bc += (int64_t)b * 2 * ncc + csc;
+  xc += (int64_t)b * 2 * ncc + csc;
+  const T* d = Jc + (int64_t)b * kJP * ncc + csc;
+#pragma unroll
+  for (int v = 0; v < 2; ++v) {
+    if (kTwo && v != part) continue;
+    const T z = fma(d[(int64_t)2 * v * ncc], sp, d[(int64_t)(2 * v + 1) * ncc] * sc);
+    bc[v * ncc] = z;
+    xc[v * ncc] = red ? z : (T)0;
+  }
 }
 
+// x_f += P x_c (prolong_value), the black cells only when post-smoothing
+// follows. rd: division by half the fine width. Grid (cells / kBlock, B).
 template <typename T>
 __global__ void __launch_bounds__(kBlock)
-k_prolong(unsigned long long* ctr, Geom Gc, Geom Gf, int B, const int* __restrict__ active,
+k_prolong(unsigned long long* ctr, Geom Gc, Geom Gf, RowDiv rd, const int* __restrict__ active,
           const T* __restrict__ xc, T* __restrict__ xf, int black_only) {
   HENRY_COUNT_LAUNCH(ctr);
-  const int ncf = Gf.ncell(), ncc = Gc.ncell();
-  const int per = black_only ? Gf.half() : ncf;   // cells corrected per sample
-  const int64_t n = (int64_t)B * per;
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n) return;
-  const int b = (int)(idx / per);
-  if (!active[b]) return;
-  const int u = (int)(idx - (int64_t)b * per);
-  const int cell = black_only ? black_cell(Gf, u) : u;
-  prolong_cell<T>(Gc, Gf, cell, xc + (int64_t)b * 2 * ncc, xf + (int64_t)b * 2 * ncf);
+  const int ncf = Gf.ncell(), half = Gf.half(), hx2 = Gf.nx >> 1;
+  const int b = blockIdx.y, u = blockIdx.x * blockDim.x + threadIdx.x;
+  if (u >= (black_only ? half : ncf) || !active[b]) return;
+  const int colour = u < half ? 1 : 0, pos = u < half ? u : u - half;
+  const int j = rd.row(pos), i = 2 * (pos - j * hx2) + ((j + colour) & 1);
+  T vp, vc;
+  prolong_value<T>(Gc, i, j, xc + (int64_t)b * 2 * Gc.ncell(), vp, vc);
+  T* x = xf + (int64_t)b * 2 * ncf + colour * half + pos;
+  x[0] += vp;
+  x[ncf] += vc;
 }
 
 // ---------------------------------------------------------------------------
@@ -1050,23 +1133,31 @@ k_vcycle_small(unsigned long long* ctr, SmallMG<T> M, int B, const int* __restri
   for (int e = threadIdx.x; e < 2 * nc; e += blockDim.x) dx[e] = xv[ks][e];
 }
 
-// Defect-correction update of the FP64 state: u += x (finest level).
+// Defect-correction update of the FP64 state: u += x (finest level), the
+// cells 2m and 2m + 1 of a row per thread. rd: division by half the width.
+// Grid (half / kBlock, B); bound by HBM on large grids.
 template <typename T>
-__global__ void k_update(unsigned long long* ctr, Geom G, int B, const int* __restrict__ active,
-                         const T* __restrict__ xvec, double* __restrict__ p, double* __restrict__ c) {
+__global__ void __launch_bounds__(kBlock)
+k_update(unsigned long long* ctr, Geom G, RowDiv rd, const int* __restrict__ active,
+         const T* __restrict__ xvec, double* __restrict__ p, double* __restrict__ c) {
   HENRY_COUNT_LAUNCH(ctr);
-  const int ncell = G.ncell();
-  const int64_t n = (int64_t)B * ncell;
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n) return;
-  const int b = (int)(idx / ncell);
-  if (!active[b]) return;
-  const int cell = (int)(idx - (int64_t)b * ncell);
-  const int j = cell / G.nx, i = cell - j * G.nx;
-  const int cs = cs_pos(i, j, G.nx, G.half());
-  const int64_t ob = (int64_t)b * 2 * ncell;
-  p[idx] += (double)xvec[ob + cs];
-  c[idx] += (double)xvec[ob + ncell + cs];
+  const int ncell = G.ncell(), half = G.half();
+  const int b = blockIdx.y, pos = blockIdx.x * blockDim.x + threadIdx.x;
+  if (pos >= half || !active[b]) return;
+  const int j = rd.row(pos);
+  // position pos of either colour's half: columns 2m + (j & 1) red, 2m + 1 - (j & 1) black
+  const T* x = xvec + (int64_t)b * 2 * ncell + pos;
+  const T pr = x[0], pk = x[half], cr = x[ncell], ck = x[ncell + half];
+  const bool odd = j & 1;
+  double2* p2 = reinterpret_cast<double2*>(p + (int64_t)b * ncell) + pos;
+  double2* c2 = reinterpret_cast<double2*>(c + (int64_t)b * ncell) + pos;
+  double2 v = *p2, w = *c2;
+  v.x += (double)(odd ? pk : pr);
+  v.y += (double)(odd ? pr : pk);
+  w.x += (double)(odd ? ck : cr);
+  w.y += (double)(odd ? cr : ck);
+  *p2 = v;
+  *c2 = w;
 }
 
 // ---------------------------------------------------------------------------
@@ -1388,13 +1479,14 @@ static __global__ void k_kry_scalars(unsigned long long* ctr, int B, int nchunk,
 
 // Vector updates of one BiCGStab iteration, one thread per entry of every
 // active sample. op 0 (start): r = rh = bt, p = v = xk = 0, scalars 1.
-// op 1: p = r + beta (p - omega v); b = p, x = 0 (preconditioner input).
-// op 2: xk += alpha y (y = x); r -= alpha v; b = r, x = 0.
+// op 1: p = r + beta (p - omega v); b = p, x = 0 (preconditioner input; on
+// the red cells x = b with half > 0, their first half-sweep).
+// op 2: xk += alpha y (y = x); r -= alpha v; b = r, x as in op 1.
 // op 3: xk += omega z (z = x); r -= omega t.
 // op 4: x = xk (the correction handed to the state update).
 template <typename T>
 __global__ void __launch_bounds__(kBlock)
-k_kry_update(unsigned long long* ctr, int n2, int B, int op, const int* __restrict__ active,
+k_kry_update(unsigned long long* ctr, int n2, int half, int B, int op, const int* __restrict__ active,
              double* __restrict__ S, T* __restrict__ r, T* __restrict__ rh, T* __restrict__ p,
              T* __restrict__ v, T* __restrict__ t, T* __restrict__ xk, T* __restrict__ bvec,
              T* __restrict__ xvec) {
@@ -1404,6 +1496,10 @@ k_kry_update(unsigned long long* ctr, int n2, int B, int op, const int* __restri
   const int b = (int)(idx / n2);
   if (!active[b]) return;
   const double* s = S + (int64_t)b * kKryS;
+  auto red = [&] {
+    const int e = (int)(idx - (int64_t)b * n2), ncell = n2 >> 1;
+    return (e < ncell ? e : e - ncell) < half;
+  };
   switch (op) {
     case 0: {
       const T bt = bvec[idx];
@@ -1417,14 +1513,14 @@ k_kry_update(unsigned long long* ctr, int n2, int B, int op, const int* __restri
     case 1: {
       const T beta = (T)s[3], omega = (T)s[2];
       const T pn = r[idx] + beta * (p[idx] - omega * v[idx]);
-      p[idx] = pn; bvec[idx] = pn; xvec[idx] = (T)0;
+      p[idx] = pn; bvec[idx] = pn; xvec[idx] = red() ? pn : (T)0;
       break;
     }
     case 2: {
       const T alpha = (T)s[1];
       xk[idx] += alpha * xvec[idx];
       const T sn = r[idx] - alpha * v[idx];
-      r[idx] = sn; bvec[idx] = sn; xvec[idx] = (T)0;
+      r[idx] = sn; bvec[idx] = sn; xvec[idx] = red() ? sn : (T)0;
       break;
     }
     case 3: {
@@ -1535,7 +1631,8 @@ __global__ void __launch_bounds__(kBlock)
 k_adj_residual(unsigned long long* ctr, Geom G, int B, const int* __restrict__ active,
                const double* __restrict__ J64, const double* __restrict__ rhs,
                const double* __restrict__ lam, double* __restrict__ res, const T* __restrict__ Jmg,
-               T* __restrict__ bvec, T* __restrict__ xvec, double* __restrict__ partial) {
+               T* __restrict__ bvec, T* __restrict__ xvec, int guess,
+               double* __restrict__ partial) {
   HENRY_COUNT_LAUNCH(ctr);
   __shared__ double sh[kBlock / 32];
   const int b = blockIdx.y;
@@ -1569,10 +1666,12 @@ k_adj_residual(unsigned long long* ctr, Geom G, int B, const int* __restrict__ a
     // right-hand side of the row-scaled transposed multigrid system
     const T* d = Jmg + (int64_t)b * kJP * n + cs;
     const T mp = (T)rp, mc = (T)rc;
-    bvec[o + cs] = d[0] * mp + d[n] * mc;
-    bvec[o + n + cs] = d[2 * n] * mp + d[3 * n] * mc;
-    xvec[o + cs] = (T)0;
-    xvec[o + n + cs] = (T)0;
+    const T bp = d[0] * mp + d[n] * mc, bc = d[2 * n] * mp + d[3 * n] * mc;
+    const bool red = guess && ((i + j) & 1) == 0;
+    bvec[o + cs] = bp;
+    bvec[o + n + cs] = bc;
+    xvec[o + cs] = red ? bp : (T)0;
+    xvec[o + n + cs] = red ? bc : (T)0;
     v = rp * rp + rc * rc;
   }
   const double s = block_sum(v, sh);

@@ -545,8 +545,9 @@ k_residual(unsigned long long* ctr, Phys P, Geom G, double vtau, ResTile tl, Res
           const int cs = cs_pos(i0 + k, j, nx, half);
           bvec[ob + cs] = bp[k];
           bvec[ob + ncell + cs] = bc[k];
-          xvec[ob + cs] = (T)0;
-          xvec[ob + ncell + cs] = (T)0;
+          const bool red = A.guess && cs < half;
+          xvec[ob + cs] = red ? bp[k] : (T)0;
+          xvec[ob + ncell + cs] = red ? bc[k] : (T)0;
         }
         if (J) {
           st_row<C>(A.qx + id, qE);

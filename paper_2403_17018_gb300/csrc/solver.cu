@@ -298,7 +298,6 @@ int Solver::ensure(int B, cudaStream_t s) {
     L.J = a + lo[k].J;
     L.b = a + lo[k].b;
     L.x = a + lo[k].x;
-    L.x2 = tb_[k] ? a + lo[k].x2 : nullptr;
     L.p = (double*)(a + lo[k].p);
     L.c = (double*)(a + lo[k].c);
     L.phi = (double*)(a + lo[k].phi);
@@ -309,6 +308,7 @@ int Solver::ensure(int B, cudaStream_t s) {
     L.dy = (double*)(a + lo[k].dy);
     L.qx = (double*)(a + lo[k].qx);
     L.qy = (double*)(a + lo[k].qy);
+    L.x2 = tb_[k] ? a + lo[k].x2 : nullptr;
   }
   c_old_ = (double*)(a + o_cold);
   p_prev_ = (double*)(a + o_pprev);
@@ -395,8 +395,11 @@ void Solver::launch_cluster(int B, int ncycles, cudaStream_t s) {
 
 // Whole hierarchy fits the shared-memory kernel, or the cluster kernel, or
 // neither (then the top levels are launched one kernel at a time).
+// guess: x of level k is the zero guess after its first red half-sweep, not
+// an iterate (only the per-operation launches make use of it: the fused
+// kernels' first red half-sweep gives the same values again).
 template <typename T>
-void Solver::enqueue_vcycle(int k, int B, cudaStream_t s) {
+void Solver::enqueue_vcycle(int k, int B, bool guess, cudaStream_t s) {
   MGLevel& L = levels_[k];
   const Geom& G = L.g;
   if (k == kc_ && kc_ > ks_ && k > 0) {
@@ -444,7 +447,7 @@ void Solver::enqueue_vcycle(int k, int B, cudaStream_t s) {
           counter_, G, C.g, B, active_, td, cfg_.nu1, (const T*)L.J, (const T*)L.b,
           (const T*)L.x, (T*)L.x2, (const T*)C.J, (T*)C.b, (T*)C.x, status_w_);
     }
-    enqueue_vcycle<T>(k - 1, B, s);
+    enqueue_vcycle<T>(k - 1, B, false, s);
     if (tu.cl) {
       cluster_cfg(tu, lc, at);
       cudaLaunchKernelEx(&lc, k_tbc_up<T>, counter_, C.g, G, B, (const int*)active_, cfg_.nu2,
@@ -458,22 +461,23 @@ void Solver::enqueue_vcycle(int k, int B, cudaStream_t s) {
     }
     return;
   }
-  const int gs = grid1((int64_t)B * G.half());
-  for (int sw = 0; sw < cfg_.nu1; ++sw)
-    for (int col = 0; col < 2; ++col)
-      k_smooth<T><<<gs, kBlock, 0, s>>>(counter_, G, B, col, active_, (const T*)L.J,
-                                       (const T*)L.b, (T*)L.x);
-  k_resid_restrict<T><<<grid1((int64_t)B * C.g.ncell()), kBlock, 0, s>>>(
-      counter_, G, C.g, B, active_, (const T*)L.J, (const T*)L.b, (const T*)L.x,
-      (const T*)C.J, (T*)C.b, (T*)C.x, cfg_.nu1 > 0);
-  enqueue_vcycle<T>(k - 1, B, s);
+  const RowDiv rd(G.nx / 2);
+  const dim3 gs(grid1(G.half()), B);
+  auto sweeps = [&](int first, int n) {
+    for (int h = first; h < 2 * n; ++h)
+      k_smooth<T><<<gs, kBlock, 0, s>>>(counter_, G, rd, h & 1, active_, (const T*)L.J, (const T*)L.b,
+                                       (T*)L.x);
+  };
+  // the guess is zero after its first red half-sweep (x_red = b_red)
+  sweeps(guess ? 1 : 0, cfg_.nu1);
+  k_resid_restrict<T><<<dim3(grid1(kRestrictThreads<T> * (int64_t)C.g.ncell()), B), kBlock, 0, s>>>(
+      counter_, G, C.g, RowDiv(C.g.nx), active_, (const T*)L.J, (const T*)L.b, (const T*)L.x,
+      (const T*)C.J, (T*)C.b, (T*)C.x, cfg_.nu1 > 0, cfg_.nu1 > 0);
+  enqueue_vcycle<T>(k - 1, B, cfg_.nu1 > 0, s);
   const int black_only = cfg_.nu2 > 0;
-  k_prolong<T><<<grid1((int64_t)B * (black_only ? G.half() : G.ncell())), kBlock, 0, s>>>(
-      counter_, C.g, G, B, active_, (const T*)C.x, (T*)L.x, black_only);
-  for (int sw = 0; sw < cfg_.nu2; ++sw)
-    for (int col = 0; col < 2; ++col)
-      k_smooth<T><<<gs, kBlock, 0, s>>>(counter_, G, B, col, active_, (const T*)L.J,
-                                       (const T*)L.b, (T*)L.x);
+  k_prolong<T><<<dim3(grid1(black_only ? G.half() : G.ncell()), B), kBlock, 0, s>>>(
+      counter_, C.g, G, rd, active_, (const T*)C.x, (T*)L.x, black_only);
+  sweeps(0, cfg_.nu2);
 }
 
 // Coarse multigrid operators at the current iterate (linearised about the
@@ -530,7 +534,7 @@ void Solver::enqueue_vcycles(int B, cudaStream_t s) {
   else if (kc_ == nl - 1 && nl > 1)
     launch_cluster<T>(B, cfg_.vcycles, s);
   else
-    for (int v = 0; v < cfg_.vcycles; ++v) enqueue_vcycle<T>(nl - 1, B, s);
+    for (int v = 0; v < cfg_.vcycles; ++v) enqueue_vcycle<T>(nl - 1, B, v == 0 && red_guess(), s);
 }
 
 // One V-cycle on the finest level's b and x (the BiCGStab preconditioner).
@@ -542,7 +546,7 @@ void Solver::enqueue_precond(int B, cudaStream_t s) {
   else if (kc_ == nl - 1 && nl > 1)
     launch_cluster<T>(B, 1, s);
   else
-    enqueue_vcycle<T>(nl - 1, B, s);
+    enqueue_vcycle<T>(nl - 1, B, red_guess(), s);
 }
 
 // krylov_iters iterations of BiCGStab on At x = bt (finest level), each
@@ -563,8 +567,9 @@ void Solver::enqueue_bicgstab(int B, cudaStream_t s) {
   T* x = (T*)F.x;
   const dim3 gd(kry_nchunk_, B);
   const int gs = (B + kBlock - 1) / kBlock;
+  const int half = red_guess() ? G.half() : 0;
   auto upd = [&](int op) {
-    k_kry_update<T><<<gv, kBlock, 0, s>>>(counter_, n2, B, op, active_, kry_S_, r, rh, p, v, t,
+    k_kry_update<T><<<gv, kBlock, 0, s>>>(counter_, n2, half, B, op, active_, kry_S_, r, rh, p, v, t,
                                           xk, b, x);
   };
   upd(0);
@@ -610,8 +615,8 @@ void Solver::enqueue_solve_update(int B, cudaStream_t s) {
   else
     enqueue_vcycles<T>(B, s);
   MGLevel& F = levels_.back();
-  k_update<T><<<grid1((int64_t)B * F.g.ncell()), kBlock, 0, s>>>(counter_, F.g, B, active_,
-                                                                 (const T*)F.x, F.p, F.c);
+  k_update<T><<<dim3(grid1(F.g.half()), B), kBlock, 0, s>>>(counter_, F.g, RowDiv(F.g.nx / 2), active_,
+                                                            (const T*)F.x, F.p, F.c);
 }
 
 template <typename T>
@@ -641,6 +646,7 @@ ResArgs Solver::res_args() const {
   a.active = active_;
   a.qx = F.qx;
   a.qy = F.qy;
+  a.guess = red_guess();
   return a;
 }
 
@@ -664,8 +670,8 @@ void Solver::launch_resjac(int B, const int* refresh, double* partial, cudaStrea
   ResArgs a = res_args();
   a.refresh = refresh;
   a.partial = partial;
-  k_residual<T, 2, true, false, false, true><<<dim3(tile_j_.warps(), B), 32, 0, s>>>(counter_, phys_, F.g, F.g.hx * F.g.hy / tau_, tile_j_,
-                                               a, (T*)F.J, (T*)F.b, (T*)F.x);
+  k_residual<T, 2, true, false, false, true><<<dim3(tile_j_.warps(), B), 32, 0, s>>>(
+      counter_, phys_, F.g, F.g.hx * F.g.hy / tau_, tile_j_, a, (T*)F.J, (T*)F.b, (T*)F.x);
 }
 
 template <typename T>
@@ -930,8 +936,6 @@ void Solver::launch_begin_step(int B, cudaStream_t s) {
 template <typename T>
 int Solver::step_t(int B, cudaStream_t s) {
   if (cfg_.loop_mode == HENRY_LOOP_GRAPH) return step_graph<T>(B, s);
-  MGLevel& F = levels_.back();
-  const Geom& G = F.g;
   launch_begin_step(B, s);
   for (;;) {
     enqueue_resjac_check<T>(B, s, false);
@@ -984,8 +988,8 @@ template <typename T>
 void Solver::launch_timed(int which, int B, cudaStream_t s) {
   MGLevel& F = levels_.back();
   if (which == 0) {
-    k_smooth<T><<<grid1((int64_t)B * F.g.half()), kBlock, 0, s>>>(
-        counter_, F.g, B, 0, active_, (const T*)F.J, (const T*)F.b, (T*)F.x);
+    k_smooth<T><<<dim3(grid1(F.g.half()), B), kBlock, 0, s>>>(
+        counter_, F.g, RowDiv(F.g.nx / 2), 0, active_, (const T*)F.J, (const T*)F.b, (T*)F.x);
   } else if (which == 2) {
     launch_resid<T>(B, s);
   } else {
@@ -1244,7 +1248,7 @@ int Solver::adjoint_t(const double* xi, const double* logk, int B, int qoi, int 
       for (;;) {
         k_adj_residual<T><<<dim3(adj_nchunk_, B), kBlock, 0, s>>>(
             counter_, G, B, active_, J64_, rhs_, lam_, res_, (const T*)F.J, (T*)F.b, (T*)F.x,
-            partial2_);
+            red_guess(), partial2_);
         k_check<false><<<(B + 7) / 8, kBlock, 0, s>>>(
             counter_, B, adj_nchunk_, G.ncell(), partial2_, 1.0, adj_rtol, 0.0, cfg_.newton_maxit,
             active_, it_step_, res0_, res_last_, status_w_, iters_w_, n_active_, check_acc_, 0.0, 0,

@@ -118,7 +118,9 @@ class Solver {
   template <typename T> void enqueue_iteration(int B, cudaStream_t s);
   template <typename T> void enqueue_rebuild(int B, cudaStream_t s);
   template <typename T> void enqueue_solve_update(int B, cudaStream_t s);
-  template <typename T> void enqueue_vcycle(int k, int B, cudaStream_t s);
+  template <typename T> void enqueue_vcycle(int k, int B, bool guess, cudaStream_t s);
+  // the guess of the multigrid solve is zero after its first red half-sweep
+  bool red_guess() const { return cfg_.nu1 > 0; }
   template <typename T> void enqueue_resjac_check(int B, cudaStream_t s, bool set_cond,
                                                   unsigned long long cond = 0);
   template <typename T> int capture_step_t(cudaGraph_t g, cudaStream_t cs, int B,

@@ -214,8 +214,8 @@ k_tb_down(unsigned long long* ctr, Geom G, Geom Gc, int B, const int* __restrict
     }
     const int csc = cs_pos(I, Jr, Gc.nx, Gc.half());
     const T* d = Jcs + csc;
-    bcs[csc] = d[0] * sp + d[ncc] * sc;
-    bcs[ncc + csc] = d[2 * ncc] * sp + d[3 * ncc] * sc;
+    bcs[csc] = fma(d[0], sp, d[ncc] * sc);
+    bcs[ncc + csc] = fma(d[2 * ncc], sp, d[3 * ncc] * sc);
     xcs[csc] = (T)0;
     xcs[ncc + csc] = (T)0;
   }
@@ -399,8 +399,8 @@ k_tbc_down(unsigned long long* ctr, Geom G, Geom Gc, int B, const int* __restric
     }
     const int csc = cs_pos(I, Jr, Gc.nx, Gc.half());
     const T* d = Jcs + csc;
-    bcs[csc] = d[0] * sp + d[ncc] * sc;
-    bcs[ncc + csc] = d[2 * ncc] * sp + d[3 * ncc] * sc;
+    bcs[csc] = fma(d[0], sp, d[ncc] * sc);
+    bcs[ncc + csc] = fma(d[2 * ncc], sp, d[3 * ncc] * sc);
     xcs[csc] = (T)0;
     xcs[ncc + csc] = (T)0;
   }
