@@ -10,6 +10,7 @@
 
 #include "kernels.cuh"
 #include "tb.cuh"
+#include "leg.cuh"
 
 namespace henry {
 
@@ -105,6 +106,13 @@ Solver::Solver(const henry_config& cfg, int nx, int ny, int nt) : cfg_(cfg), nt_
     tbd_[k] = make_tb_tile(geoms_[k], cfg_.nu1, 1, kTbTileX, kTbTileY, 20, tsize_);
     tbu_[k] = make_tb_tile(geoms_[k], cfg_.nu2, 0, kTbTileX, kTbTileY, 16, tsize_);
   }
+  // one launch per leg (k_leg) on the other batched FP32 levels
+  leg_.assign(geoms_.size(), 0);
+  for (size_t k = 1; k < geoms_.size(); ++k) {
+    const bool fused = (int)k <= ks_ || ((int)k <= kc_ && kc_ > ks_);
+    leg_[k] = cfg_.mg_fusion && !fused && !tb_[k] && tsize_ == sizeof(float) && cfg_.nu1 == 2 &&
+              cfg_.nu2 == 2;
+  }
 }
 
 Solver::~Solver() { free_all(); }
@@ -188,6 +196,10 @@ int Solver::ensure(int B, cudaStream_t s) {
       CK(raise_smem_limit((const void*)k_vcycle_small<double>, small_smem_bytes(Md)));
   }
   for (size_t k = 1; k < levels_.size(); ++k) {
+    if (leg_[k]) {
+      CK(raise_smem_limit((const void*)k_leg<false>, kLegSmem));
+      CK(raise_smem_limit((const void*)k_leg<true>, kLegSmem));
+    }
     if (!tb_[k]) continue;
     const bool f32 = tsize_ == sizeof(float);
     const TbTile& d = tbd_[k];
@@ -308,7 +320,9 @@ int Solver::ensure(int B, cudaStream_t s) {
     L.dy = (double*)(a + lo[k].dy);
     L.qx = (double*)(a + lo[k].qx);
     L.qy = (double*)(a + lo[k].qy);
-    L.x2 = tb_[k] ? a + lo[k].x2 : nullptr;
+    // k_leg's second iterate: the face fluxes, which a rebuild writes and
+    // reads before the cycles start, leave their place (8 bytes a cell)
+    L.x2 = tb_[k] ? (void*)(a + lo[k].x2) : leg_[k] ? (void*)L.qx : nullptr;
   }
   c_old_ = (double*)(a + o_cold);
   p_prev_ = (double*)(a + o_pprev);
@@ -463,6 +477,25 @@ void Solver::enqueue_vcycle(int k, int B, bool guess, cudaStream_t s) {
   }
   const RowDiv rd(G.nx / 2);
   const dim3 gs(grid1(G.half()), B);
+  if constexpr (sizeof(T) == sizeof(float)) {
+    const LegTile t = make_leg_tile(G, B);
+    if (leg_[k] && leg_pays(G, B, t)) {
+      // pre-sweeps + restriction (x -> x2), the coarse levels, prolongation +
+      // post-sweeps (x2 -> x); k_leg starts after the first red half-sweep
+      if (!guess)
+        k_smooth<T><<<gs, kBlock, 0, s>>>(counter_, G, rd, 0, active_, (const T*)L.J, (const T*)L.b,
+                                         (T*)L.x);
+      const dim3 gl(t.blocks(), B);
+      k_leg<false><<<gl, 32 * kLegWarps, kLegSmem, s>>>(counter_, G, C.g, t, active_, (const T*)L.J, (const T*)L.b,
+                                        (const T*)L.x, (T*)L.x2, nullptr, (const T*)C.J, (T*)C.b,
+                                        (T*)C.x);
+      enqueue_vcycle<T>(k - 1, B, true, s);
+      k_leg<true><<<gl, 32 * kLegWarps, kLegSmem, s>>>(counter_, G, C.g, t, active_, (const T*)L.J, (const T*)L.b,
+                                       (const T*)L.x2, (T*)L.x, (const T*)C.x, nullptr, nullptr,
+                                       nullptr);
+      return;
+    }
+  }
   auto sweeps = [&](int first, int n) {
     for (int h = first; h < 2 * n; ++h)
       k_smooth<T><<<gs, kBlock, 0, s>>>(counter_, G, rd, h & 1, active_, (const T*)L.J, (const T*)L.b,

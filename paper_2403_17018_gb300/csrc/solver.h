@@ -204,6 +204,7 @@ class Solver {
   int kc_ = 0;                // top multigrid level handled by k_vcycle_cluster
   int cl_ = 1;                // blocks per cluster (one cluster per sample)
   std::vector<char> tb_;      // per multigrid level: legs temporally blocked
+  std::vector<char> leg_;     // per multigrid level: a launch per leg (k_leg)
   std::vector<TbTile> tbd_, tbu_;   // tiles of the down (halo 2 nu1 + 1) and up legs
   // CUDA graph of one time step (HENRY_LOOP_GRAPH), rebuilt when B changes
   cudaGraphExec_t step_exec_ = nullptr;
