@@ -1297,7 +1297,9 @@ int Solver::adjoint_t(const double* xi, const double* logk, int B, int qoi, int 
       // Eq. e_recharge_of_param: the inflow of step st carries (1 + sin(pi t / 40)), t = st tau
       const double qfac =
           cfg_.field_model == 1 ? 1.0 + sin(3.14159265358979323846 * st * tau_ / 40.0) : 1.0;
-      k_adj_sens<<<grid1((int64_t)n), kBlock, 0, s>>>(counter_, phys_, G, tau_, qfac, B, F.p, F.c,
+      const SensConst sens = {G.hx * G.hy / tau_, G.hy * phys_.D / G.hx, G.hx * phys_.D / G.hy,
+                              2.0 * G.hy * phys_.D / G.hx, 2.0 * G.hy / (phys_.mu * G.hx)};
+      k_adj_sens<<<grid1((int64_t)n), kBlock, 0, s>>>(counter_, phys_, G, sens, qfac, B, F.p, F.c,
                                                       c_old_,
                                                       F.phi, F.K, F.tx, F.dx, F.ty, F.dy, lam_, gK_,
                                                       gphi_, gq_);
