@@ -388,7 +388,7 @@ def roofline(ctx, flush, peaks, fp64_tflops):
             "fp64_pipe": {"achieved_tflops": round(tf, 4), "peak_tflops": round(fp64_tflops, 4),
                           "frac": round(tf / fp64_tflops, 4),
                           "peak_source": "measured in this run (henry_probe_fp64)"},
-            "second": {"kernel": "k_resjac<double> (FP64 residual + Jacobian, level 3), cold",
+            "second": {"kernel": "k_residual<double> (FP64 residual + Jacobian, level 3), cold",
                        "ms_per_launch": round(ms2, 5),
                        "achieved_gbs": round(by2 / (ms2 / 1e3) / 1e9, 1),
                        "fp64_tflops": round(fl2 / (ms2 / 1e3) / 1e12, 4),
@@ -416,7 +416,7 @@ def streaming(flush, hbm, fp64_tflops):
             "smoother": kernel_line(ctx, 0, 0, 20, flush, hbm, fp64_tflops, T,
                                     f"k_smooth<{tname}> red half-sweep, 1024x512 x 16, cold"),
             "residual_jacobian": kernel_line(ctx, 0, 1, 10, flush, hbm, fp64_tflops, T,
-                                             f"k_resjac<{tname}>, 1024x512 x 16, cold")}
+                                             f"k_residual<{tname}> (with J), 1024x512 x 16, cold")}
         ctx.close()
     return out
 
