@@ -999,8 +999,8 @@ k_resid_restrict(unsigned long long* ctr, Geom Gf, Geom Gc, RowDiv rd, const int
   xc += (int64_t)b * 2 * ncc + csc;
   const T* d = Jc + (int64_t)b * kJP * ncc + csc;
 #pragma unroll
-  for (int v = 0; v < 2; ++v) {
-    if (kTwo && v != part) continue;
+  for (int m = 0; m < (kTwo ? 1 : 2); ++m) {
+    const int v = kTwo ? part : m;
     const T z = fma(d[(int64_t)2 * v * ncc], sp, d[(int64_t)(2 * v + 1) * ncc] * sc);
     bc[v * ncc] = z;
     xc[v * ncc] = red ? z : (T)0;
