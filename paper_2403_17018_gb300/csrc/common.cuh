@@ -16,7 +16,8 @@ constexpr int kMaxCoarseUnknowns = 64;
 
 #define HENRY_COUNT_LAUNCH(ctr)                                                        \
   do {                                                                                 \
-    if (ctr && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)                 \
+    if (ctr && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 &&               \
+        threadIdx.y == 0)                                                              \
       atomicAdd((unsigned long long*)(ctr), 1ULL);                                     \
   } while (0)
 
