@@ -25,10 +25,20 @@ __device__ __forceinline__ double stat_sum(double v, double* sh) {
   return t;
 }
 
+// Sum of squared deviations from the mean, given the sums f1 of deviations
+// and f2 of squared deviations from a shift close to the mean and inv = 1 / n.
+// Rounding of the difference must not leave a negative variance (a NaN stays).
+__device__ __forceinline__ double centred_m2(double f1, double f2, double inv) {
+  const double v = fma(-f1 * inv, f1, f2);
+  return v < 0.0 ? 0.0 : v;
+}
+
 // Moments of one QoI (blockIdx.x) over the valid samples of the batch, two
 // passes: out[0] = n, then mean_f, m2_f, mean_d, m2_d [kNQ] of g = q_fine
-// and d = q_fine - q_coarse. m2 = sum (g - mean)^2 - (sum (g - mean))^2 / n,
-// whose second term removes the rounding of the mean. Grid kNQ blocks: 600
+// and d = q_fine - q_coarse. The first pass sums the distances from the first
+// valid sample, so that the mean of a constant batch (counted cells, empty
+// boxes) is its value and its variance zero, exactly; the second the
+// deviations from that mean (centred_m2). Grid kNQ blocks: 600
 // samples take 8 us, where one block that ran Welford's update (two
 // divisions per sample and QoI) took 387 us.
 __global__ void __launch_bounds__(kStatThreads)
@@ -37,7 +47,20 @@ k_level_stats(unsigned long long* ctr, int B, const double* __restrict__ qf,
               double* __restrict__ out) {
   HENRY_COUNT_LAUNCH(ctr);
   __shared__ double sh[kStatThreads / 32];
+  __shared__ int first;
   const int k = blockIdx.x;
+  if (threadIdx.x == 0) first = B;
+  __syncthreads();
+  int b0 = threadIdx.x;
+  while (b0 < B && status && status[b0] != 0) b0 += kStatThreads;
+  b0 = __reduce_min_sync(0xffffffffu, b0);
+  if ((threadIdx.x & 31) == 0 && b0 < B) atomicMin(&first, b0);
+  __syncthreads();
+  double xf = 0.0, xd = 0.0;                // the first valid sample's g and d
+  if (first < B) {
+    xf = qf[(int64_t)first * kNQ + k];
+    xd = qc ? xf - qc[(int64_t)first * kNQ + k] : xf;
+  }
   double cnt = 0.0, sf = 0.0, sd = 0.0;
   auto each = [&](auto&& f) {
     for (int b = threadIdx.x; b < B; b += kStatThreads) {
@@ -48,13 +71,13 @@ k_level_stats(unsigned long long* ctr, int B, const double* __restrict__ qf,
   };
   each([&](double g, double d) {
     cnt += 1.0;
-    sf += g;
-    sd += d;
+    sf += g - xf;
+    if (qc) sd += d - xd;
   });
   const double n = stat_sum(cnt, sh);
   const double inv = n > 0.0 ? 1.0 / n : 0.0;
-  const double mf = stat_sum(sf, sh) * inv;
-  const double md = qc ? stat_sum(sd, sh) * inv : mf;
+  const double mf = fma(stat_sum(sf, sh), inv, xf);
+  const double md = qc ? fma(stat_sum(sd, sh), inv, xd) : mf;
   double f1 = 0.0, f2 = 0.0, d1 = 0.0, d2 = 0.0;
   each([&](double g, double d) {
     const double e = g - mf;
@@ -78,9 +101,9 @@ k_level_stats(unsigned long long* ctr, int B, const double* __restrict__ qf,
   if (threadIdx.x == 0) {
     if (k == 0) out[0] = n;
     out[1 + k] = fma(f1, inv, mf);
-    out[1 + kNQ + k] = fma(-f1 * inv, f1, f2);
+    out[1 + kNQ + k] = centred_m2(f1, f2, inv);
     out[1 + 2 * kNQ + k] = fma(d1, inv, md);
-    out[1 + 3 * kNQ + k] = fma(-d1 * inv, d1, d2);
+    out[1 + 3 * kNQ + k] = centred_m2(d1, d2, inv);
   }
 }
 
@@ -106,8 +129,9 @@ __device__ __forceinline__ void chan_merge(Moments& a, const Moments& b) {
 // the running state held in device memory. A block takes 32 cells and G
 // groups of consecutive samples; each thread sums the deviations and their
 // squares of its cell over its group's valid samples about a shift, the mean
-// of the group's first (up to 8) valid samples, so that nothing cancels: three
-// FP64 instructions per sample (and quantity). The groups are merged by a
+// of eight samples from the group's first valid one on (which stands in for
+// missing and failed ones, summed in pairs: the shift of a constant cell is
+// its value), so that nothing cancels: three FP64 instructions per sample (and quantity). The groups are merged by a
 // fixed tree (Chan). 600 samples of 8192 cells: 1028 us with a thread per cell running
 // Welford's update, 61 us so.
 constexpr int kShift = 8;
@@ -130,21 +154,27 @@ __global__ void k_field_stats(unsigned long long* ctr, int nx, int ny, int B,
     const int ccell = (j >> 1) * (nx / 2) + (i >> 1);
     const double* pf = cf + cell;
     const double* pc = cc ? cc + ccell : nullptr;
-    double kf = 0.0, kd = 0.0, c = 0.0;
-    int bs = b0;                              // the first valid sample, then 8 from there
+    double kf = 0.0, kd = 0.0;
+    int bs = b0;                              // the first valid sample
     while (bs < b1 && status && status[bs] != 0) ++bs;
+    if (bs < b1) {
+      double g[kShift], u[kShift];
 #pragma unroll
-    for (int u = 0; u < kShift; ++u) {
-      const int b = bs + u < b1 ? bs + u : b1 - 1;
-      if (bs + u >= b1 || (status && status[b] != 0)) continue;
-      const double g = pf[(int64_t)b * ncell];
-      kf += g;
-      if (pc) kd += g - pc[(int64_t)b * ncc];
-      c += 1.0;
+      for (int m = 0; m < kShift; ++m) {
+        const int b = bs + m < b1 && (!status || status[bs + m] == 0) ? bs + m : bs;
+        g[m] = pf[(int64_t)b * ncell];
+        u[m] = pc ? g[m] - pc[(int64_t)b * ncc] : 0.0;
+      }
+#pragma unroll
+      for (int w = kShift / 2; w > 0; w >>= 1)
+#pragma unroll
+        for (int m = 0; m < w; ++m) {
+          g[m] += g[m + w];
+          u[m] += u[m + w];
+        }
+      kf = g[0] * (1.0 / kShift);
+      kd = u[0] * (1.0 / kShift);
     }
-    const double cw = c == kShift ? 1.0 / kShift : c > 0.0 ? 1.0 / c : 0.0;
-    kf *= cw;
-    kd *= cw;
     double f1 = 0.0, f2 = 0.0, d1 = 0.0, d2 = 0.0;
     int cnt = 0;
 #pragma unroll 8
@@ -165,8 +195,8 @@ __global__ void k_field_stats(unsigned long long* ctr, int nx, int ny, int B,
     }
     if (cnt > 0) {
       const double w = 1.0 / (double)cnt;
-      f = {(double)cnt, fma(f1, w, kf), fma(-f1 * w, f1, f2)};
-      d = pc ? Moments{(double)cnt, fma(d1, w, kd), fma(-d1 * w, d1, d2)} : f;
+      f = {(double)cnt, fma(f1, w, kf), centred_m2(f1, f2, w)};
+      d = pc ? Moments{(double)cnt, fma(d1, w, kd), centred_m2(d1, d2, w)} : f;
     }
   }
   mom[y * 32 + x] = f;
