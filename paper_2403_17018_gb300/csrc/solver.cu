@@ -3,14 +3,13 @@
 
 #include <cstdio>
 #include <cstring>
-#include <map>
-#include <mutex>
 #include <string>
 #include <utility>
 
 #include "kernels.cuh"
 #include "tb.cuh"
 #include "leg.cuh"
+#include "smem_limit.h"
 
 namespace henry {
 
@@ -161,20 +160,16 @@ int Solver::debug_copy(int mg_level, int what, void* dst, int64_t bytes) const {
   return HENRY_OK;
 }
 
-// The dynamic shared-memory limit of a kernel is an attribute of the
-// function in the device's context, shared by every solver of the process:
-// it is only ever raised, to the largest size any solver needs, and outside
-// stream capture (from ensure()), so that no solver's graph capture can meet
-// a limit lowered by another solver.
+// Raises a kernel's dynamic shared-memory limit on the current device;
+// called outside stream capture (from ensure()).
 static cudaError_t raise_smem_limit(const void* fn, size_t smem) {
-  static std::mutex mu;
-  static std::map<const void*, size_t> cur;
-  std::lock_guard<std::mutex> lock(mu);
-  size_t& c = cur[fn];
-  if (smem <= c || smem <= 48 * 1024) return cudaSuccess;
-  const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess) c = smem;
-  return e;
+  static SmemLimits limits;
+  int device = 0;
+  const cudaError_t e = cudaGetDevice(&device);
+  if (e != cudaSuccess) return e;
+  return limits.raise(device, fn, smem, [](const void* f, size_t bytes) {
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  });
 }
 
 int Solver::ensure(int B, cudaStream_t s) {
