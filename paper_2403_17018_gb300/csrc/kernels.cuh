@@ -376,14 +376,16 @@ __global__ void k_check(unsigned long long* ctr, int B, int nchunk, int ncell,
 // long as its chain of dependent FP64 instructions and L2 reads whatever the
 // level's size (16 samples of the 64x32 hierarchy, FP64: 76 us per rebuild;
 // 128x64 x 64, FP32: 87 us).
-constexpr int kMaxLevels = 12;
+// A hierarchy's coarsest grid keeps at least 8 cells and its finest has fewer
+// than 2^31, a quarter per level: 8 * 4^13 = 2^29.
+constexpr int kMaxHierarchy = 14;
 
 struct CoarseStates {
   int nl;                           // levels; the finest is nl - 1
-  Geom g[kMaxLevels];
-  double* c[kMaxLevels];
-  double* qx[kMaxLevels];
-  double* qy[kMaxLevels];
+  Geom g[kMaxHierarchy];
+  double* c[kMaxHierarchy];
+  double* qx[kMaxHierarchy];
+  double* qy[kMaxHierarchy];
 };
 
 constexpr int kRestrictDepth = 5;   // levels that one launch descends
@@ -569,11 +571,11 @@ k_coarse_inv(unsigned long long* ctr, Geom G, int B, const int* __restrict__ act
 template <typename T>
 struct CoarseOps {
   CoarseStates st;
-  const double *phi[kMaxLevels], *K[kMaxLevels], *tx[kMaxLevels], *dx[kMaxLevels], *ty[kMaxLevels],
-      *dy[kMaxLevels];
-  T* J[kMaxLevels];
-  double vtau[kMaxLevels];           // cell volume / time step
-  int first[kMaxLevels];             // first block of the level
+  const double *phi[kMaxHierarchy], *K[kMaxHierarchy], *tx[kMaxHierarchy], *dx[kMaxHierarchy], *ty[kMaxHierarchy],
+      *dy[kMaxHierarchy];
+  T* J[kMaxHierarchy];
+  double vtau[kMaxHierarchy];           // cell volume / time step
+  int first[kMaxHierarchy];             // first block of the level
 };
 
 template <typename T>
@@ -1038,6 +1040,7 @@ k_prolong(unsigned long long* ctr, Geom Gc, Geom Gf, RowDiv rd, const int* __res
 // memory hold their mbarrier.
 // ---------------------------------------------------------------------------
 constexpr int kSmallCells = 512;   // largest level the shared-memory kernel accepts
+constexpr int kMaxLevels = 12;     // levels of the fused kernels' tables
 
 template <typename T>
 struct SmallMG {
