@@ -459,25 +459,61 @@ k_restrict_states(unsigned long long* ctr, const __grid_constant__ CoarseStates 
 }
 
 // Explicit inverse of the coarsest system (the direct coarse solve of the
-// multigrid, section 2.3) by one block: Gauss-Jordan elimination with partial
-// pivoting by rows, one barrier per pivot. Every warp finds the pivot row and
-// the pivot's reciprocal for itself, and every element of the next matrix is
-// formed from the last one's in another buffer: row k and the pivot row
-// interchanged, the new row k divided by the pivot (its own column becoming 1
-// / pivot), f times it subtracted from the others (their column k becoming -f
-// / pivot). The column interchanges that undo the row pivots (last pivot
-// first) are folded into the output index. Unknown order 2*cell + var, cell
-// natural; the inverse is stored transposed, Ainv^T[v][u] at v*n + u, so that
-// the coarse solve x = Ainv b reads it with lanes over u. The arithmetic is
-// the multigrid type T (the coarse solve is part of the preconditioner): one
-// n^3 elimination per operator rebuild turns each coarse solve into one
-// parallel matrix-vector product instead of 2n dependent substitution steps.
-// Bound by the chain of n reciprocals and multiply-adds.
+// multigrid, section 2.3) by one block: in-place Gauss-Jordan elimination with
+// partial pivoting by rows, two barriers per pivot. Warp 0 finds the pivot row
+// (by the magnitudes' bits: an FP64 comparison costs as much as an FP64
+// multiplication), keeps the multipliers of column k, interchanges row k and
+// the pivot row and divides the new row k by the pivot (its own column becoming
+// 1 / pivot); then all warps subtract f times that row from the others (their
+// column k becoming -f / pivot). The column interchanges that undo the row
+// pivots (last pivot first) are folded into the output index. Unknown order
+// 2*cell + var, cell natural; the inverse is stored transposed, Ainv^T[v][u]
+// at v*n + u, so that the coarse solve x = Ainv b reads it with lanes over u.
+// The arithmetic is the multigrid type T (the coarse solve is part of the
+// preconditioner): one n^3 elimination per operator rebuild turns each coarse
+// solve into one parallel matrix-vector product instead of 2n dependent
+// substitution steps. Bound by the chain of n reciprocals on small systems and
+// by the FP64 pipe on large ones, n^2 / 32 instructions a pivot: whatever more
+// than one warp repeats, and a product formed once per element instead of once
+// per column, counts there. FP64, us: 16 unknowns x 16 samples 18.5, 60 x 16
+// 148, 60 x 1024 466; with one barrier per pivot, the search and the reciprocal
+// in every warp and the pivot row's product in every element 26.7, 258 and
+// 1531; with three barriers and FP64 comparisons 30.8, 226 and 720.
 constexpr int kInvThreads = 128;
+constexpr int kInvThreadsMost = 256;
+
+// Threads of the inverse's block (n unknowns, B blocks): 256 shorten the
+// passes over a large matrix as long as the blocks have the SMs to
+// themselves. FP64, us with 128 / 256: 60 unknowns x 16 197 / 140, x 304 215 /
+// 178, x 1024 465 / 535; 16 unknowns x 304 18.6 / 20.5, x 1024 23 / 45.
+inline int inv_threads(int n, int B) { return n > 24 && B <= 2 * 152 ? kInvThreadsMost : kInvThreads; }
 
 template <typename T>
 __host__ __device__ inline size_t coarse_inv_smem_bytes(int n) {
-  return 2 * (size_t)n * (n + 1) * sizeof(T) + 2 * (size_t)n * sizeof(int);
+  return ((size_t)n * (n + 1) + n) * sizeof(T) + 2 * (size_t)n * sizeof(int);
+}
+
+// |v| as an integer of the same order; a NaN comes before everything.
+__device__ __forceinline__ long long magnitude_key(double v) {
+  const long long b = __double_as_longlong(v) & 0x7fffffffffffffffll;
+  return b > 0x7ff0000000000000ll ? -1 : b;
+}
+__device__ __forceinline__ int magnitude_key(float v) {
+  const int b = __float_as_int(v) & 0x7fffffff;
+  return b > 0x7f800000 ? -1 : b;
+}
+
+// The lane-wise (key, row) pairs' largest key, lowest row among equals.
+__device__ __forceinline__ int warp_argmax(int key, int row) {
+  const int m = __reduce_max_sync(0xffffffffu, key);
+  return __reduce_min_sync(0xffffffffu, key == m ? row : 0x7fffffff);
+}
+__device__ __forceinline__ int warp_argmax(long long key, int row) {
+  const int hi = (int)(key >> 32);
+  const int mh = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned lo = hi == mh ? (unsigned)key : 0u;
+  const unsigned ml = __reduce_max_sync(0xffffffffu, lo);
+  return __reduce_min_sync(0xffffffffu, hi == mh && lo == ml ? row : 0x7fffffff);
 }
 
 template <typename T>
@@ -485,8 +521,8 @@ __device__ __forceinline__ void coarse_inverse(const Geom& G, const T* Jb, T* __
                                                unsigned char* smem) {
   const int nc = G.ncell(), n = 2 * nc, half = G.half(), ld = n + 1;
   T* A = (T*)smem;
-  T* Y = A + n * ld;
-  int* pv = (int*)(Y + n * ld);         // pivot row of each step
+  T* fcol = A + n * ld;                 // multipliers of column k, after the interchange
+  int* pv = (int*)(fcol + n);           // pivot row of each step
   int* qcol = pv + n;                   // output column -> eliminated column
   const int l = threadIdx.x & 31;
   for (int e = threadIdx.x; e < n * ld; e += blockDim.x) A[e] = (T)0;
@@ -508,36 +544,71 @@ __device__ __forceinline__ void coarse_inverse(const Geom& G, const T* Jb, T* __
   __syncthreads();
   const int step_r = blockDim.x / n, step_c = blockDim.x - step_r * n;
   const int r0 = threadIdx.x / n, c0 = threadIdx.x - r0 * n;
+  // two elements at a time hide the loads' latency; many blocks of FP32 are bound by
+  // the instructions instead (60 unknowns x 1024, us: 291 in pairs, 240 without)
+  const bool pairs = sizeof(T) == 8 || n <= 32 || blockDim.x > kInvThreads;
   for (int k = 0; k < n; ++k) {
-    // pivot: largest |A[r][k]|, r >= k, lowest index on ties
-    T bv = (T)-1;
-    int br = k;
-    for (int r = k + l; r < n; r += 32) {
-      const T v = fabs(A[r * ld + k]);
-      if (v > bv) { bv = v; br = r; }
-    }
+    if (threadIdx.x < 32) {
+      // pivot: largest |A[r][k]|, r >= k, lowest index on ties
+      auto bv = magnitude_key((T)NAN);
+      int br = k;
+      for (int r = k + l; r < n; r += 32) {
+        const auto v = magnitude_key(A[r * ld + k]);
+        if (v > bv) { bv = v; br = r; }
+      }
+      br = warp_argmax(bv, br);
+      const T d = A[br * ld + k];
+      T a[2], o[2], f[2];               // pivot row, row k, column k after the interchange
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const T ov = __shfl_xor_sync(0xffffffffu, bv, o);
-      const int orr = __shfl_xor_sync(0xffffffffu, br, o);
-      if (ov > bv || (ov == bv && orr < br)) { bv = ov; br = orr; }
+      for (int m = 0; m < 2; ++m) {
+        const int c = l + 32 * m;
+        if (c >= n) continue;
+        a[m] = A[br * ld + c];
+        o[m] = A[k * ld + c];
+        f[m] = A[(c == br ? k : c) * ld + k];
+      }
+      const T rinv = d != (T)0 ? (T)1 / d : (T)0;
+      if (l == 0) pv[k] = br;
+      __syncwarp();                     // all is read before the rows change
+#pragma unroll
+      for (int m = 0; m < 2; ++m) {
+        const int c = l + 32 * m;
+        if (c >= n) continue;
+        fcol[c] = f[m];
+        if (br != k) A[br * ld + c] = o[m];
+        A[k * ld + c] = (c == k ? (T)1 : a[m]) * rinv;
+      }
     }
-    const T d = A[br * ld + k];
-    const T rinv = d != (T)0 ? (T)1 / d : (T)0;
-    if (threadIdx.x == 0) pv[k] = br;
+    __syncthreads();
     int r = r0, c = c0;
+    while (pairs && r < n) {
+      T v[2], f[2], p[2];
+      int at[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        at[u] = r < n && r != k ? r * ld + c : -1;
+        if (at[u] >= 0) {
+          v[u] = c == k ? (T)0 : A[at[u]];
+          f[u] = fcol[r];
+          p[u] = A[k * ld + c];
+        }
+        r += step_r;
+        c += step_c;
+        if (c >= n) { c -= n; ++r; }
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        if (at[u] >= 0) A[at[u]] = fma(-f[u], p[u], v[u]);
+    }
     while (r < n) {
-      const int src = r == br ? k : r;
-      const T prow = (c == k ? (T)1 : A[br * ld + c]) * rinv;
-      const T v = c == k ? (T)0 : A[src * ld + c];
-      Y[r * ld + c] = r == k ? prow : fma(-A[src * ld + k], prow, v);
+      if (r != k) {
+        const T v = c == k ? (T)0 : A[r * ld + c];
+        A[r * ld + c] = fma(-fcol[r], A[k * ld + c], v);
+      }
       r += step_r;
       c += step_c;
       if (c >= n) { c -= n; ++r; }
     }
-    T* s = A;
-    A = Y;
-    Y = s;
     __syncthreads();
   }
   // column c of the inverse is column q(c) of the eliminated matrix, with
@@ -555,7 +626,7 @@ __device__ __forceinline__ void coarse_inverse(const Geom& G, const T* Jb, T* __
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kInvThreads)
+__global__ void __launch_bounds__(kInvThreadsMost)
 k_coarse_inv(unsigned long long* ctr, Geom G, int B, const int* __restrict__ active,
              const T* __restrict__ J, T* __restrict__ AinvT, const int* __restrict__ refresh) {
   HENRY_COUNT_LAUNCH(ctr);
@@ -608,7 +679,7 @@ __device__ __forceinline__ void coarse_jac_cell(const Phys& P, const CoarseOps<T
 // dependent pivots then runs beside the other levels' cells), the blocks from
 // first[k] on level k. Dynamic shared memory coarse_inv_smem_bytes<T>(n).
 template <typename T>
-__global__ void __launch_bounds__(kInvThreads)
+__global__ void __launch_bounds__(kInvThreadsMost)
 k_coarse_ops(unsigned long long* ctr, Phys P, const __grid_constant__ CoarseOps<T> M, int B,
              const int* __restrict__ active, T* __restrict__ AinvT, const int* __restrict__ refresh) {
   HENRY_COUNT_LAUNCH(ctr);

@@ -520,6 +520,7 @@ void Solver::enqueue_coarse_ops(int B, cudaStream_t s, const int* refresh, bool 
   CoarseOps<T> M = {};
   M.st.nl = nl;
   int blocks = B;
+  const int n0 = 2 * levels_[0].g.ncell(), threads = inv_threads(n0, B);
   for (int k = 0; k < nl; ++k) {
     const MGLevel& L = levels_[k];
     M.st.g[k] = L.g;
@@ -535,7 +536,7 @@ void Solver::enqueue_coarse_ops(int B, cudaStream_t s, const int* refresh, bool 
     M.J[k] = (T*)L.J;
     M.vtau[k] = L.g.hx * L.g.hy / tau_;
     M.first[k] = blocks;
-    if (k > 0 && k < nl - 1) blocks += (int)(((int64_t)B * L.g.ncell() + kInvThreads - 1) / kInvThreads);
+    if (k > 0 && k < nl - 1) blocks += (int)(((int64_t)B * L.g.ncell() + threads - 1) / threads);
   }
   for (int top = nl - 1; top >= 1;) {
     const int depth = top < kRestrictDepth ? top : kRestrictDepth;
@@ -543,14 +544,14 @@ void Solver::enqueue_coarse_ops(int B, cudaStream_t s, const int* refresh, bool 
     k_restrict_states<<<grid1(cells), kBlock, 0, s>>>(counter_, M.st, top, depth, B, active_, refresh);
     top -= depth;
   }
-  k_coarse_ops<T><<<blocks, kInvThreads, coarse_inv_smem_bytes<T>(2 * levels_[0].g.ncell()), s>>>(
+  k_coarse_ops<T><<<blocks, threads, coarse_inv_smem_bytes<T>(n0), s>>>(
       counter_, phys_, M, B, active_, with_inv ? (T*)cinv_ : nullptr, refresh);
 }
 
 template <typename T>
 void Solver::enqueue_coarse_inv(int B, cudaStream_t s, const int* refresh) {
   const int n = 2 * levels_[0].g.ncell();
-  k_coarse_inv<T><<<B, kInvThreads, coarse_inv_smem_bytes<T>(n), s>>>(
+  k_coarse_inv<T><<<B, inv_threads(n, B), coarse_inv_smem_bytes<T>(n), s>>>(
       counter_, levels_[0].g, B, active_, (const T*)levels_[0].J, (T*)cinv_, refresh);
 }
 
