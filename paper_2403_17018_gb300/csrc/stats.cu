@@ -130,8 +130,9 @@ __device__ __forceinline__ void chan_merge(Moments& a, const Moments& b) {
 // groups of consecutive samples; each thread sums the deviations and their
 // squares of its cell over its group's valid samples about a shift, the mean
 // of eight samples from the group's first valid one on (which stands in for
-// missing and failed ones, summed in pairs: the shift of a constant cell is
-// its value), so that nothing cancels: three FP64 instructions per sample (and quantity). The groups are merged by a
+// failed ones, summed in pairs: the shift of a constant cell is its value) or
+// of fewer where the group has no more, so that nothing cancels: three FP64
+// instructions per sample (and quantity). The groups are merged by a
 // fixed tree (Chan). 600 samples of 8192 cells: 1028 us with a thread per cell running
 // Welford's update, 61 us so.
 constexpr int kShift = 8;
@@ -157,7 +158,20 @@ __global__ void k_field_stats(unsigned long long* ctr, int nx, int ny, int B,
     double kf = 0.0, kd = 0.0;
     int bs = b0;                              // the first valid sample
     while (bs < b1 && status && status[bs] != 0) ++bs;
-    if (bs < b1) {
+    if (bs < b1 && b1 - bs < kShift) {        // a short group: its mean, from the first one's distance
+      const double x0 = pf[(int64_t)bs * ncell], y0 = pc ? x0 - pc[(int64_t)bs * ncc] : 0.0;
+      int c = 1;
+      for (int b = bs + 1; b < b1; ++b) {
+        if (status && status[b] != 0) continue;
+        const double g = pf[(int64_t)b * ncell];
+        kf += g - x0;
+        if (pc) kd += (g - pc[(int64_t)b * ncc]) - y0;
+        ++c;
+      }
+      const double w = c > 1 ? 1.0 / (double)c : 0.0;
+      kf = fma(kf, w, x0);
+      kd = fma(kd, w, y0);
+    } else if (bs < b1) {
       double g[kShift], u[kShift];
 #pragma unroll
       for (int m = 0; m < kShift; ++m) {
