@@ -137,7 +137,8 @@ __device__ __forceinline__ void chan_merge(Moments& a, const Moments& b) {
 // Welford's update, 61 us so.
 constexpr int kShift = 8;
 
-__global__ void k_field_stats(unsigned long long* ctr, int nx, int ny, int B,
+__global__ void __launch_bounds__(1024)
+k_field_stats(unsigned long long* ctr, int nx, int ny, int B,
                               const double* __restrict__ cf, const double* __restrict__ cc,
                               const int* __restrict__ status, int64_t* __restrict__ n,
                               double* __restrict__ mean_f, double* __restrict__ m2_f,
@@ -251,7 +252,8 @@ __device__ __forceinline__ long long order_key(double v) {
   return b ^ ((b >> 63) & 0x7fffffffffffffffll);
 }
 
-__global__ void k_field_exceed(unsigned long long* ctr, int ncell, int B,
+__global__ void __launch_bounds__(1024)
+k_field_exceed(unsigned long long* ctr, int ncell, int B,
                                const double* __restrict__ c, const int* __restrict__ status,
                                double threshold, int64_t* __restrict__ count) {
   HENRY_COUNT_LAUNCH(ctr);
