@@ -450,10 +450,14 @@ int henry_level_info(const henry_ctx* ctx, int level, int* nx, int* ny, int* nt,
  * mg_level (0 = coarsest). what: 0 J [B][24][ncell] (colour-split planes:
  * inverse diagonal block, W, E, S, N blocks row-scaled by it, diagonal
  * block),
- * 1 b, 2 x ([B][2][ncell], colour-split), 3 p, 4 c, 5 phi, 6 K ([B][ncell],
- * natural), 7..10 face constants tx, dx, ty, dy, 11..12 face fluxes of the
- * linearisation point qx (east faces; the right side in the last column),
- * qy (north faces), 13 the BiCGStab scalars of the last defect correction
+ * 1 b, 2 x ([B][2][ncell], colour-split; on the finest level, after a solve,
+ * the last residual's right-hand side and the guess that would go with it,
+ * zero or, with nu1 > 0, b on the red cells), 3 p, 4 c, 5 phi, 6 K ([B][ncell],
+ * natural), 7..10 face constants tx, dx, ty, dy, 11..12 face fluxes qx (east
+ * faces; the right side in the last column), qy (north faces): on the finest
+ * level of the state that the last residual was evaluated at, on the others
+ * of the iterate that the operators were last rebuilt at, 13 the BiCGStab
+ * scalars of the last defect correction
  * ([B][8] FP64: rho, alpha, omega, beta, then unused; only with
  * krylov_iters > 0). Element size is 4 bytes for J, b, x with FP32
  * multigrid, else 8. Copies min(bytes, size) bytes

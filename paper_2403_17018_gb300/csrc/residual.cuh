@@ -573,4 +573,35 @@ k_residual(unsigned long long* ctr, Phys P, Geom G, double vtau, ResTile tl, Res
   }
 }
 
+// Face fluxes of the state (p, c), as the residual-only form evaluates them
+// (which does not store them: only a rebuild reads them): qx of the east faces,
+// the right side in the last column, qy of the north faces. For diagnostics.
+static __global__ void k_face_fluxes(Phys P, Geom G, int B, const double* __restrict__ p,
+                                     const double* __restrict__ c, const double* __restrict__ tx,
+                                     const double* __restrict__ ty, double* __restrict__ qx,
+                                     double* __restrict__ qy) {
+  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= (int64_t)B * G.ncell()) return;
+  const int cell = (int)(idx % G.ncell()), j = cell / G.nx, i = cell - j * G.nx;
+  auto value = [&](int64_t at) {
+    CellV v = {p[at], c[at], 0.0, 0.0};
+    cell_values(P, v);
+    return v;
+  };
+  const CellV L = value(idx);
+  const double hd = 0.5 * P.drho, hdg = hd * P.g * G.hy;
+  double q, m, s;
+  if (i < G.nx - 1) {
+    res_face<false>(P, L, value(idx + 1), tx[idx], 0.0, 0.0, q, m, s);
+  } else {
+    const double h = P.Ly - (j + 0.5) * G.hy;
+    const CellV sea = {P.drho * P.g * h, 1.0, P.rho0 + P.drho, P.rho0 + P.drho};
+    res_face<false>(P, L, sea, tx[idx], 0.0, 0.0, q, m, s);
+  }
+  qx[idx] = q;
+  q = 0.0;
+  if (j < G.ny - 1) res_face<true>(P, L, value(idx + G.nx), ty[idx], 0.0, hdg, q, m, s);
+  qy[idx] = q;
+}
+
 }  // namespace henry

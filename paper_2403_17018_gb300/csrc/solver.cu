@@ -156,6 +156,10 @@ int Solver::debug_copy(int mg_level, int what, void* dst, int64_t bytes) const {
                            n * 8, n * 8, n * 8, n * 8, n * 8, n * 8, n * 8, n * 8};
   const size_t nb = (size_t)bytes < size[what] ? (size_t)bytes : size[what];
   CK(cudaDeviceSynchronize());
+  if ((what == 11 || what == 12) && resid_last_ && mg_level == (int)levels_.size() - 1) {
+    k_face_fluxes<<<grid1((int64_t)n), kBlock>>>(phys_, L.g, cap_, L.p, L.c, L.tx, L.ty, L.qx, L.qy);
+    CK(cudaGetLastError());
+  }
   CK(cudaMemcpy(dst, src[what], nb, cudaMemcpyDefault));
   return HENRY_OK;
 }
@@ -247,7 +251,7 @@ int Solver::ensure(int B, cudaStream_t s) {
     lo[k].J = take(kJP * n * tsize_);
     lo[k].b = take(2 * n * tsize_);
     lo[k].x = take(2 * n * tsize_);
-    lo[k].x2 = take(tb_[k] ? 2 * n * tsize_ : 0);
+    lo[k].x2 = take(tb_[k] || leg_[k] ? 2 * n * tsize_ : 0);   // second iterate of a leg
     lo[k].p = take(n * 8);
     lo[k].c = take(n * 8);
     lo[k].phi = take(n * 8);
@@ -315,9 +319,7 @@ int Solver::ensure(int B, cudaStream_t s) {
     L.dy = (double*)(a + lo[k].dy);
     L.qx = (double*)(a + lo[k].qx);
     L.qy = (double*)(a + lo[k].qy);
-    // k_leg's second iterate: the face fluxes, which a rebuild writes and
-    // reads before the cycles start, leave their place (8 bytes a cell)
-    L.x2 = tb_[k] ? (void*)(a + lo[k].x2) : leg_[k] ? (void*)L.qx : nullptr;
+    L.x2 = tb_[k] || leg_[k] ? a + lo[k].x2 : nullptr;
   }
   c_old_ = (double*)(a + o_cold);
   p_prev_ = (double*)(a + o_pprev);
@@ -924,6 +926,7 @@ int Solver::setup_t(const double* xi, const double* logk, int B, cudaStream_t s)
                                                                 iters_w_, step_);
   k_set_int<<<1, 32, 0, s>>>(counter_, keep_, cfg_.jac_keep);
   CK(cudaGetLastError());
+  resid_last_ = cfg_.jac_lag > 0;
   return HENRY_OK;
 }
 
@@ -1308,6 +1311,7 @@ int Solver::adjoint_t(const double* xi, const double* logk, int B, int qoi, int 
                                       gphi_, gq_, dq_dxi);
   if (dq_dlogk) CK(cudaMemcpyAsync(dq_dlogk, gK_, n * 8, cudaMemcpyDeviceToDevice, s));
   k_copy_int<<<grid1(B), kBlock, 0, s>>>(counter_, B, status_w_, status, 0);
+  resid_last_ = false;
   CK(cudaGetLastError());
   return HENRY_OK;
 }
