@@ -135,12 +135,15 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   return s;
 }
 
-// Tiling of k_residual (residual.cuh): lpr lanes share a row of a warp (C columns each), gpw row groups
-// per warp, R rows per group; ntx x nty warps cover a sample.
+// Tiling of k_residual (residual.cuh): lpr lanes share a row of a warp (C
+// columns each), gpw row groups per warp, R rows per group; ntx x nty tiles
+// cover a sample, a warp each, or `split` warps that share the rows.
 struct ResTile {
-  int lpr, gpw, R, ntx, nty;
-  __host__ __device__ int warps() const { return ntx * nty; }
+  int lpr, gpw, R, ntx, nty, split;
+  __host__ __device__ int tiles() const { return ntx * nty; }
 };
+
+constexpr int kResSplit = 4;   // bands of rows, and most warps, of a tile that warps may share
 
 // rows 0 selects the tile height from the grid alone (never from the batch:
 // the partial sums that decide convergence keep their order whatever the
@@ -152,19 +155,56 @@ struct ResTile {
 // with 8, 717 with 16. With the Jacobian (FP32): 32x16 x 1 16 with 2 rows, 27
 // with 4; 128x64 x 64 94 with 2, 89 with 4, 80 with 8, but x 16 25, 29, 47;
 // 1024x512 x 16 978 with 8, 967 with 16.
+//
+// The lanes per row are those whose warps do the least work, counted in FP64
+// instructions, which cost a warp the same however many lanes are active: per
+// row and column 34 (with the Jacobian about 90), per group of rows the south
+// faces again, per lpr rows the west face of a tile's first column. On widths
+// that are a multiple of 32 C columns those are all 32. Residual only (FP32),
+// us: 80x24 cells x 1024 322 with tiles of 32 and 8 lanes, 212 with five of 8;
+// 192x160 x 256 852 with 32 and 16, 660 with three of 16.
 __host__ inline ResTile make_res_tile(int nx, int ny, int C, int rows, bool jac) {
-  ResTile t;
-  const int lanes = (nx + C - 1) / C;
-  t.lpr = lanes < 32 ? lanes : 32;
-  t.gpw = 32 / t.lpr;
-  t.ntx = (lanes + 31) / 32;
+  const int lanes = (nx + C - 1) / C, cell = jac ? 90 : 34, face = jac ? 35 : 13;
   const int64_t ncell = (int64_t)nx * ny;
   if (rows <= 0)
     rows = jac ? (ncell <= 4096 ? 2 : (ncell <= 65536 ? 4 : (ncell <= 262144 ? 8 : 16)))
                : (ncell <= 4096 ? 2 : (ncell <= 65536 ? 4 : (ncell <= 262144 ? 16 : 8)));
-  const int most = (ny + t.gpw - 1) / t.gpw;
-  t.R = rows < most ? rows : most;
-  t.nty = (ny + t.gpw * t.R - 1) / (t.gpw * t.R);
+  ResTile best = {};
+  int64_t least = -1;
+  for (int lpr = lanes < 32 ? lanes : 32; lpr >= 1; --lpr) {
+    ResTile t = {};
+    t.lpr = lpr;
+    t.gpw = 32 / lpr;
+    const int all = (ny + t.gpw - 1) / t.gpw;   // rows per group if a tile covered the height
+    t.R = rows < all ? rows : all;
+    t.ntx = (lanes + lpr - 1) / lpr;
+    t.nty = (all + t.R - 1) / t.R;
+    t.split = 1;
+    const int64_t cost = (int64_t)t.tiles() * (t.R * C * cell + C * face +
+                                               (t.ntx > 1 ? (t.R + lpr - 1) / lpr * face : 0));
+    if (least < 0 || cost < least) {
+      least = cost;
+      best = t;
+    }
+  }
+  return best;
+}
+
+// Warps that share a tile of B samples' grids, where the kernel allows it
+// (its sum goes over kResSplit bands of rows either way, so that the batch
+// leaves it as it is): those whose waves over `slots` resident warps take the
+// fewest rows, a third of a row more for the south faces. Residual only, FP64,
+// 512x256 cells, us with a warp per tile / so: x 1 102 / 34 (four), x 4 102 / 57
+// (four), x 8 124 / 105 (two), x 16 175 / 175 (one), x 64 743 / 693 (two).
+__host__ inline ResTile split_res_tile(ResTile t, int B, int slots) {
+  int64_t least = -1;
+  for (int s = 1; s <= kResSplit && t.R % kResSplit == 0; s *= 2) {
+    const int64_t waves = ((int64_t)t.tiles() * B * s + slots - 1) / slots, cost = waves * (3 * t.R / s + 1);
+    if (least < 0 || cost < least) {
+      least = cost;
+      t.split = s;
+    }
+  }
   return t;
 }
 

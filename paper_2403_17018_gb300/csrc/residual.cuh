@@ -11,12 +11,13 @@
 //    walks R rows; faces between its own columns stay in registers, the face
 //    to the next lane's column is passed by shuffle, the north face becomes
 //    the next row's south face. Only a tile's first row (south) and, on
-//    grids wider than 32 C columns, its first column (west; all rows of it
+//    grids of several tiles in x, its first column (west; all rows of it
 //    in one pass, a row per lane) are evaluated twice;
 //  * the unit of scheduling is one warp (a block of 32 threads, no barrier,
 //    no shared memory), so a small batch spreads over all SMs: 16 samples of
 //    64x32 cells are 128 to 256 blocks, where a 256-thread tile per sample
-//    kept 16 SMs busy;
+//    kept 16 SMs busy. Tall tiles, which a large batch wants, may be shared by
+//    the warps of a block (SPLIT);
 //  * the densities and rho c are formed once per cell; upwinding tests the
 //    sign bit of the flux (integer pipe); the FP32 Jacobian takes its face
 //    constants from FP32 copies instead of converting them.
@@ -153,16 +154,17 @@ __device__ __forceinline__ void own_face(double ck, double cd, double k1, double
 // operator, b = -Dinv R and x = 0 in the colour-split layout. The solver's
 // residual-only form takes the old time level's storage terms as arrays.
 // OWN: full pressure, face constants and storage from phi and K. V: vector
-// loads (nx even and every array 16-byte aligned). Grid (warps of a sample,
-// B), 32 threads.
+// loads (nx even and every array 16-byte aligned). SPLIT: tl.split warps share
+// a tile. Grid (tiles of a sample, B), 32 threads (times tl.split).
 //
 // Registers: a warp's registers come from its scheduler's 16,384, so 128 per
 // thread keep 4 warps per scheduler, 168 keep 3 and 255 keep 2; the bounds
 // below take the step that the kernel reaches without spilling.
 constexpr int res_min_blocks(int C, bool J, bool own) { return J ? 8 : (own ? 12 : C == 4 ? 8 : 16); }
+constexpr int kResSplitSlots = 152 * res_min_blocks(4, false, false);   // warps resident
 
-template <typename T, int C, bool J, bool NAT, bool OWN, bool V>
-__global__ void __launch_bounds__(32, res_min_blocks(C, J, OWN))
+template <typename T, int C, bool J, bool NAT, bool OWN, bool V, bool SPLIT = false>
+__global__ void __launch_bounds__(SPLIT ? 32 * kResSplit : 32, res_min_blocks(C, J, OWN) / (SPLIT ? kResSplit : 1))
 k_residual(unsigned long long* ctr, Phys P, Geom G, double vtau, ResTile tl, ResArgs A,
            T* __restrict__ Jm, T* __restrict__ bvec, T* __restrict__ xvec) {
   HENRY_COUNT_LAUNCH(ctr);
@@ -172,11 +174,14 @@ k_residual(unsigned long long* ctr, Phys P, Geom G, double vtau, ResTile tl, Res
   if (A.active && !A.active[b]) return;
   if (A.refresh && !A.refresh[b]) return;
   const int nx = G.nx, ny = G.ny, ncell = G.ncell(), half = G.half();
-  const int lane = threadIdx.x;
+  const int lane = threadIdx.x & 31;
   const int grp = lane / tl.lpr, col = lane - grp * tl.lpr;
   const int by = blockIdx.x / tl.ntx, bx = blockIdx.x - by * tl.ntx;
-  const int i0 = (bx * 32 + col) * C;
-  const int j0 = (by * tl.gpw + grp) * tl.R;
+  const int i0 = (bx * tl.lpr + col) * C;
+  // SPLIT: rows per band, this warp's first band and rows
+  const int h = SPLIT ? tl.R / kResSplit : 1, band0 = SPLIT ? (threadIdx.x >> 5) * (kResSplit / tl.split) : 0;
+  const int rows = SPLIT ? tl.R / tl.split : tl.R;
+  const int j0 = (by * tl.gpw + grp) * tl.R + band0 * h;
   const bool thr = grp < tl.gpw && i0 < nx;
   const bool last = i0 + C >= nx;                            // owns the right side
   const bool edge = thr && !last && col == tl.lpr - 1;       // east neighbour in the next tile
@@ -255,11 +260,12 @@ k_residual(unsigned long long* ctr, Phys P, Geom G, double vtau, ResTile tl, Res
       }
     }
   }
+  __shared__ double band_sum[SPLIT ? kResSplit : 1][32];
   double v = 0.0;
   double w0 = 0.0, w1 = 0.0, edgeP = 0.0;
   FaceJ<T> wJ{};
 #pragma unroll 1
-  for (int r = 0; r < tl.R; ++r) {
+  for (int r = 0; r < rows; ++r) {
     const int j = j0 + r;
     const bool cv = thr && j < ny;
     const int64_t id = o + (int64_t)j * nx;
@@ -271,12 +277,12 @@ k_residual(unsigned long long* ctr, Phys P, Geom G, double vtau, ResTile tl, Res
     const int rl = r % tl.lpr;
     if (rl == 0) {
       const int jw = j0 + r + col;
-      if (grp < tl.gpw && r + col < tl.R && jw < ny) {
+      if (grp < tl.gpw && r + col < rows && jw < ny) {
         if (bx == tl.ntx - 1) {
           edgeP = P.Ly - (jw + 0.5) * G.hy;
           if (!J) edgeP = P.drho * P.g * edgeP;
         }
-        const int64_t e = (int64_t)b * ncell + (int64_t)jw * nx + bx * 32 * C;
+        const int64_t e = o - col * C + (int64_t)jw * nx;
         if (bx == 0) {
           w0 = A.qin[(int64_t)b * ny + jw];
           w1 = dcoL * A.phi[e];
@@ -565,6 +571,17 @@ k_residual(unsigned long long* ctr, Phys P, Geom G, double vtau, ResTile tl, Res
         jS[k] = jN[k];
       }
     }
+    if (SPLIT && (r + 1) % h == 0) {
+      band_sum[band0 + r / h][lane] = v;
+      v = 0.0;
+    }
+  }
+  if (SPLIT) {   // the tile's sum, in the order of its bands
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    v = band_sum[0][lane];
+#pragma unroll
+    for (int m = 1; m < kResSplit; ++m) v += band_sum[m][lane];
   }
   if (A.partial) {
 #pragma unroll

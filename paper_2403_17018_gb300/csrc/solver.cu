@@ -83,7 +83,9 @@ Solver::Solver(const henry_config& cfg, int nx, int ny, int nt) : cfg_(cfg), nt_
   res_cols_ = fine.nx % 4 == 0 && fine.ncell() > 4096 ? 4 : 2;
   tile_r_ = make_res_tile(fine.nx, fine.ny, res_cols_, cfg.res_rows, false);
   tile_j_ = make_res_tile(fine.nx, fine.ny, 2, cfg.res_rows, true);
-  nchunk_ = cfg.jac_lag ? tile_r_.warps() : tile_j_.warps();
+  nchunk_ = cfg.jac_lag ? tile_r_.tiles() : tile_j_.tiles();
+  // tall default tiles of the residual-only kernel are shared by warps where the batch is small
+  res_split_ = res_cols_ == 4 && cfg.res_rows == 0 && tile_r_.R == 16;
   ks_ = 0;
   kc_ = 0;
   for (size_t k = 0; k < geoms_.size(); ++k) {
@@ -278,7 +280,8 @@ int Solver::ensure(int B, cudaStream_t s) {
   const size_t o_step = take(8);
   const size_t o_qin = take((size_t)F.ny * Bz * 8);
   const size_t o_qin0 = take((size_t)F.ny * Bz * 8);
-  const size_t o_part = take((size_t)nchunk_ * Bz * 8);
+  const int nsum = tile_r_.tiles() > tile_j_.tiles() ? tile_r_.tiles() : tile_j_.tiles();
+  const size_t o_part = take((size_t)nsum * Bz * 8);   // (kernel timing runs either form)
   const size_t o_qoi = take((size_t)qoi_chunks() * kQoiSums * Bz * 8);
   const size_t o_res0 = take(Bz * 8);
   const size_t o_resl = take(Bz * 8);
@@ -687,10 +690,12 @@ void Solver::launch_resid(int B, cudaStream_t s) {
   MGLevel& F = levels_.back();
   ResArgs a = res_args();
   a.partial = partial_;
-  auto kern = res_cols_ == 4 ? k_residual<T, 4, false, false, false, true>
-                             : k_residual<T, 2, false, false, false, true>;
-  kern<<<dim3(tile_r_.warps(), B), 32, 0, s>>>(counter_, phys_, F.g, F.g.hx * F.g.hy / tau_, tile_r_,
-                                               a, (T*)F.J, (T*)F.b, (T*)F.x);
+  auto kern = res_split_      ? k_residual<T, 4, false, false, false, true, true>
+              : res_cols_ == 4 ? k_residual<T, 4, false, false, false, true>
+                               : k_residual<T, 2, false, false, false, true>;
+  const ResTile t = res_split_ ? split_res_tile(tile_r_, B, kResSplitSlots) : tile_r_;
+  kern<<<dim3(t.tiles(), B), 32 * t.split, 0, s>>>(counter_, phys_, F.g, F.g.hx * F.g.hy / tau_, t, a,
+                                                   (T*)F.J, (T*)F.b, (T*)F.x);
 }
 
 // Residual and operators of the finest level, for the samples that ask for
@@ -701,7 +706,7 @@ void Solver::launch_resjac(int B, const int* refresh, double* partial, cudaStrea
   ResArgs a = res_args();
   a.refresh = refresh;
   a.partial = partial;
-  k_residual<T, 2, true, false, false, true><<<dim3(tile_j_.warps(), B), 32, 0, s>>>(
+  k_residual<T, 2, true, false, false, true><<<dim3(tile_j_.tiles(), B), 32, 0, s>>>(
       counter_, phys_, F.g, F.g.hx * F.g.hy / tau_, tile_j_, a, (T*)F.J, (T*)F.b, (T*)F.x);
 }
 
@@ -1267,7 +1272,7 @@ int Solver::adjoint_t(const double* xi, const double* logk, int B, int qoi, int 
       k_activate<<<grid1(B), kBlock, 0, s>>>(counter_, B, status_w_, active_, it_step_);
       // operators of step st: J (multigrid type, every level) and exact FP64 J
       launch_resjac<T>(B, nullptr, nullptr, s);
-      k_residual<double, 2, true, true, false, true><<<dim3(tile_j_.warps(), B), 32, 0, s>>>(
+      k_residual<double, 2, true, true, false, true><<<dim3(tile_j_.tiles(), B), 32, 0, s>>>(
           counter_, phys_, G, G.hx * G.hy / tau_, tile_j_, res_args(), J64_, res_, nullptr);
       enqueue_coarse_ops<T>(B, s, nullptr, false);
       for (size_t k = 0; k < levels_.size(); ++k)
@@ -1355,7 +1360,7 @@ cudaError_t launch_residual_jacobian(const Phys& P, const Geom& G, double tau, i
                        : k_residual<double, 2, false, true, true, true>)
                   : (J ? k_residual<double, 1, true, true, true, false>
                        : k_residual<double, 1, false, true, true, false>);
-  kern<<<dim3(t.warps(), B), 32, 0, s>>>(nullptr, P, G, G.hx * G.hy / tau, t, a, J, R, nullptr);
+  kern<<<dim3(t.tiles(), B), 32, 0, s>>>(nullptr, P, G, G.hx * G.hy / tau, t, a, J, R, nullptr);
   return cudaGetLastError();
 }
 

@@ -199,6 +199,7 @@ class Solver {
   int* keep_ = nullptr;       // device flag: operators kept across steps (k_check)
   int nchunk_ = 0;            // residual partial sums per sample (k_check)
   int res_cols_ = 2;          // columns per thread of the residual-only kernel
+  bool res_split_ = false;    // its tiles may be shared by warps
   bool resid_last_ = false;   // the last residual stored no face fluxes (see debug_copy)
   ResTile tile_r_{}, tile_j_{};   // tiling of k_residual without and with the Jacobian
   int ks_ = 0;                // top multigrid level handled by k_vcycle_small
