@@ -121,20 +121,17 @@ struct FaceD {
 };
 
 // Interior face. t = A K_f/(mu d), dco = A phi_f D / d, gd = g e_y d.
-// q is the area-weighted face flux A q.n: computed from p unless Q_GIVEN, in
-// which case the caller supplies it (coarse multigrid levels linearise about
-// the restricted fine-level flux field) and the pressures are not used.
+// q is the area-weighted face flux A q.n, supplied by the caller (coarse
+// multigrid levels linearise about the restricted fine-level flux field).
 // VERT: a vertical (south-north) face, the only kind with a gravity term;
 // horizontal faces skip it (and its derivative) instead of multiplying by a
 // zero gd.
-template <typename JT, bool WANT_J, bool Q_GIVEN, bool VERT>
-__device__ __forceinline__ void face_flux(const Phys& P, double pL, double cL, double pU, double cU,
-                                          double t, double dco, double gd, double& q,
-                                          double& Fm, double& Fs, FaceD<JT>& J) {
+template <typename JT, bool WANT_J, bool VERT>
+__device__ __forceinline__ void face_flux(const Phys& P, double cL, double cU, double t, double dco,
+                                          double gd, double q, double& Fm, double& Fs, FaceD<JT>& J) {
   const double rL = P.rho0 + P.drho * cL;
   const double rU = P.rho0 + P.drho * cU;
   const double rbar = 0.5 * (rL + rU);
-  if (!Q_GIVEN) q = VERT ? -t * ((pU - pL) + (0.5 * P.drho) * (cL + cU) * gd) : -t * (pU - pL);
   const bool up = q >= 0.0;
   const double rup = up ? rL : rU;
   const double rcup = up ? rL * cL : rU * cU;
@@ -169,48 +166,23 @@ __device__ __forceinline__ void face_flux(const Phys& P, double pL, double cL, d
   }
 }
 
-// Right side (x = Lx, outward +x): flux from P to the seawater boundary and
-// its derivatives with respect to (p_P, c_P). tR = 2 A K_P / (mu hx),
-// dco = 2 A phi_P D / hx, pb = reduced Dirichlet pressure.
-template <typename JT, bool WANT_J, bool Q_GIVEN>
-__device__ __forceinline__ void right_face(const Phys& P, double p, double c, double tR, double dco,
-                                           double pb, double& q, double& Fm, double& Fs, JT* jd) {
-  const double rho = P.rho0 + P.drho * c;
-  const double rho1 = P.rho0 + P.drho;
-  if (!Q_GIVEN) q = -tR * (pb - p);
-  const bool up = q >= 0.0;
-  const double rup = up ? rho : rho1;
-  const double rcup = up ? rho * c : rho1;
-  const double rb = 0.5 * (rho + rho1);
-  Fm = q * rup;
-  Fs = q * rcup - dco * rb * (1.0 - c);
-  if (WANT_J) {
-    jd[0] = (JT)(tR * rup);
-    jd[1] = (JT)(up ? q * P.drho : 0.0);
-    jd[2] = (JT)(tR * rcup);
-    jd[3] = (JT)((up ? q * (rho + P.drho * c) : 0.0) - dco * 0.5 * P.drho * (1.0 - c) + dco * rb);
-  }
-}
-
 // Inputs of one cell's residual/Jacobian evaluation, gathered by the caller.
 struct CellIn {
-  double p, c, c_old, phi, K;       // own values (K used on the right side only)
-  double pW, cW, pE, cE, pS, cS, pN, cN;
+  double c, c_old, phi, K;          // own values (K used on the right side only)
+  double cW, cE, cS, cN;
   double tW, dW, tE, dE, tS, dS, tN, dN;   // face constants (valid where the face exists)
   double qin;                        // left inflow velocity of this row (i == 0)
-  double qW, qE, qS, qN;             // face fluxes A q.n (qE: right side when i == nx-1);
-                                     // outputs, or inputs when Q_GIVEN
+  double qW, qE, qS, qN;             // face fluxes A q.n (qE: right side when i == nx-1)
   bool hasW, hasE, hasS, hasN;       // interior faces
-  double y;                          // cell-centre y (right boundary pressure)
 };
 
 // Residual (FP64) and, optionally, the 20 Jacobian entries of one cell;
 // vtau = cell volume / time step:
 // J[0..3] = dR_P/du_P, J[4..7] W, J[8..11] E, J[12..15] S, J[16..19] N;
 // each block (pp, pc, cp, cc), row = equation, column = variable.
-template <typename JT, bool WANT_J, bool Q_GIVEN = false>
+template <typename JT, bool WANT_J>
 __device__ __forceinline__ void cell_residual(const Phys& P, const Geom& G, double vtau,
-                                              CellIn& in, double& Rp, double& Rc, JT* J) {
+                                              const CellIn& in, double& Rp, double& Rc, JT* J) {
   const double vt = vtau * in.phi;
   const double rho = P.rho0 + P.drho * in.c;
   const double rho_o = P.rho0 + P.drho * in.c_old;
@@ -227,7 +199,7 @@ __device__ __forceinline__ void cell_residual(const Phys& P, const Geom& G, doub
   const double gdy = P.g * G.hy;
   // west face: L = W, U = P; contributes -F to P
   if (in.hasW) {
-    face_flux<JT, WANT_J, Q_GIVEN, false>(P, in.pW, in.cW, in.p, in.c, in.tW, in.dW, 0.0, in.qW, Fm, Fs, d);
+    face_flux<JT, WANT_J, false>(P, in.cW, in.c, in.tW, in.dW, 0.0, in.qW, Fm, Fs, d);
     Rp -= Fm;
     Rc -= Fs;
     if (WANT_J) {
@@ -245,7 +217,7 @@ __device__ __forceinline__ void cell_residual(const Phys& P, const Geom& G, doub
   }
   // east face: L = P, U = E; contributes +F to P
   if (in.hasE) {
-    face_flux<JT, WANT_J, Q_GIVEN, false>(P, in.p, in.c, in.pE, in.cE, in.tE, in.dE, 0.0, in.qE, Fm, Fs, d);
+    face_flux<JT, WANT_J, false>(P, in.c, in.cE, in.tE, in.dE, 0.0, in.qE, Fm, Fs, d);
     Rp += Fm;
     Rc += Fs;
     if (WANT_J) {
@@ -258,8 +230,6 @@ __device__ __forceinline__ void cell_residual(const Phys& P, const Geom& G, doub
     const double rho1 = P.rho0 + P.drho;
     const double tR = 2.0 * A * in.K / (P.mu * G.hx);
     const double dco = 2.0 * A * in.phi * P.D / G.hx;
-    const double pb = P.drho * P.g * (P.Ly - in.y);   // reduced pressure
-    if (!Q_GIVEN) in.qE = -tR * (pb - in.p);
     const double q = in.qE;
     const bool up = q >= 0.0;
     const double rup = up ? rho : rho1;
@@ -277,7 +247,7 @@ __device__ __forceinline__ void cell_residual(const Phys& P, const Geom& G, doub
   }
   // south face: L = S, U = P (e = +y); contributes -F
   if (in.hasS) {
-    face_flux<JT, WANT_J, Q_GIVEN, true>(P, in.pS, in.cS, in.p, in.c, in.tS, in.dS, gdy, in.qS, Fm, Fs, d);
+    face_flux<JT, WANT_J, true>(P, in.cS, in.c, in.tS, in.dS, gdy, in.qS, Fm, Fs, d);
     Rp -= Fm;
     Rc -= Fs;
     if (WANT_J) {
@@ -287,7 +257,7 @@ __device__ __forceinline__ void cell_residual(const Phys& P, const Geom& G, doub
   }
   // north face: L = P, U = N; contributes +F
   if (in.hasN) {
-    face_flux<JT, WANT_J, Q_GIVEN, true>(P, in.p, in.c, in.pN, in.cN, in.tN, in.dN, gdy, in.qN, Fm, Fs, d);
+    face_flux<JT, WANT_J, true>(P, in.c, in.cN, in.tN, in.dN, gdy, in.qN, Fm, Fs, d);
     Rp += Fm;
     Rc += Fs;
     if (WANT_J) {
@@ -299,14 +269,13 @@ __device__ __forceinline__ void cell_residual(const Phys& P, const Geom& G, doub
 
 // Gather the stencil of cell (i, j) from natural-layout arrays of one sample.
 // tx/dx hold east-face constants, ty/dy north-face constants.
-__device__ __forceinline__ void gather_cell(const Geom& G, int i, int j, const double* __restrict__ p,
+__device__ __forceinline__ void gather_cell(const Geom& G, int i, int j,
                                             const double* __restrict__ c, const double* __restrict__ phi,
                                             const double* __restrict__ K, const double* __restrict__ tx,
                                             const double* __restrict__ dx, const double* __restrict__ ty,
                                             const double* __restrict__ dy, CellIn& in) {
   const int nx = G.nx;
   const int id = j * nx + i;
-  in.p = p[id];
   in.c = c[id];
   in.phi = phi[id];
   in.hasW = i > 0;
@@ -314,11 +283,10 @@ __device__ __forceinline__ void gather_cell(const Geom& G, int i, int j, const d
   in.hasS = j > 0;
   in.hasN = j < G.ny - 1;
   in.K = in.hasE ? 0.0 : K[id];
-  in.y = (j + 0.5) * G.hy;
-  if (in.hasW) { in.pW = p[id - 1]; in.cW = c[id - 1]; in.tW = tx[id - 1]; in.dW = dx[id - 1]; }
-  if (in.hasE) { in.pE = p[id + 1]; in.cE = c[id + 1]; in.tE = tx[id]; in.dE = dx[id]; }
-  if (in.hasS) { in.pS = p[id - nx]; in.cS = c[id - nx]; in.tS = ty[id - nx]; in.dS = dy[id - nx]; }
-  if (in.hasN) { in.pN = p[id + nx]; in.cN = c[id + nx]; in.tN = ty[id]; in.dN = dy[id]; }
+  if (in.hasW) { in.cW = c[id - 1]; in.tW = tx[id - 1]; in.dW = dx[id - 1]; }
+  if (in.hasE) { in.cE = c[id + 1]; in.tE = tx[id]; in.dE = dx[id]; }
+  if (in.hasS) { in.cS = c[id - nx]; in.tS = ty[id - nx]; in.dS = dy[id - nx]; }
+  if (in.hasN) { in.cN = c[id + nx]; in.tN = ty[id]; in.dN = dy[id]; }
 }
 
 // Random fields at the point (x, y) (frame y in [0, Ly]) for one sample's

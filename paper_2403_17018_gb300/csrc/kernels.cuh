@@ -658,8 +658,8 @@ __device__ __forceinline__ void coarse_jac_cell(const Phys& P, const CoarseOps<T
   const int64_t o = (int64_t)b * ncell;
   const double *c = M.st.c[k], *qx = M.st.qx[k], *qy = M.st.qy[k];
   CellIn in;
-  gather_cell(G, i, j, c + o, c + o, M.phi[k] + o, M.K[k] + o, M.tx[k] + o, M.dx[k] + o, M.ty[k] + o,
-              M.dy[k] + o, in);   // (the fluxes are given: no pressures)
+  gather_cell(G, i, j, c + o, M.phi[k] + o, M.K[k] + o, M.tx[k] + o, M.dx[k] + o, M.ty[k] + o,
+              M.dy[k] + o, in);
   in.c_old = in.c;
   in.qin = 0.0;
   in.qE = qx[o + cell];
@@ -668,7 +668,7 @@ __device__ __forceinline__ void coarse_jac_cell(const Phys& P, const CoarseOps<T
   in.qS = in.hasS ? qy[o + cell - G.nx] : 0.0;
   double Rp, Rc;
   T Jc[20];
-  cell_residual<T, true, true>(P, G, M.vtau[k], in, Rp, Rc, Jc);
+  cell_residual<T, true>(P, G, M.vtau[k], in, Rp, Rc, Jc);
   T* Jb = M.J[k] + (int64_t)b * kJP * ncell + cs_pos(i, j, G.nx, G.half());
   T d[4];
   store_operator<T>(Jb, ncell, Jc, d);

@@ -653,12 +653,6 @@ void Solver::enqueue_solve_update(int B, cudaStream_t s) {
                                                             (const T*)F.x, F.p, F.c);
 }
 
-template <typename T>
-void Solver::enqueue_iteration(int B, cudaStream_t s) {
-  enqueue_rebuild<T>(B, s);
-  enqueue_solve_update<T>(B, s);
-}
-
 // Inputs of k_residual on the finest level's workspace.
 ResArgs Solver::res_args() const {
   const MGLevel& F = levels_.back();

@@ -115,7 +115,6 @@ class Solver {
   template <typename T> void enqueue_vcycles(int B, cudaStream_t s);
   template <typename T> void enqueue_precond(int B, cudaStream_t s);
   template <typename T> void enqueue_bicgstab(int B, cudaStream_t s);
-  template <typename T> void enqueue_iteration(int B, cudaStream_t s);
   template <typename T> void enqueue_rebuild(int B, cudaStream_t s);
   template <typename T> void enqueue_solve_update(int B, cudaStream_t s);
   template <typename T> void enqueue_vcycle(int k, int B, bool guess, cudaStream_t s);
