@@ -978,6 +978,21 @@ struct RowDiv {
   }
 };
 
+// Launch of n threads per sample: the fewest blocks of at most kBlock threads,
+// as equal as whole warps allow. 272 positions are two blocks of 160 (32x17
+// nodes x 256, a solve of the vertex-centred variant: 52.7 ms; 58.3 with a
+// block of 256 and one with 16 of its 256 threads in use, 57.0 with the
+// samples' positions in one flat index).
+struct RowGrid {
+  dim3 grid;
+  int threads;
+  RowGrid(int64_t n, int B) {
+    const int64_t blocks = (n + kBlock - 1) / kBlock;
+    grid = dim3((unsigned)blocks, (unsigned)B);
+    threads = (int)(((n + blocks - 1) / blocks + 31) & ~31);
+  }
+};
+
 // One red (colour 0) or black (colour 1) half-sweep of point-block
 // Gauss-Seidel on every sample. Grid (half / kBlock, B). Bound by HBM on
 // large grids (FP32, 1024x512 x 16: 56 us for the 369 MB it moves) and by the

@@ -476,15 +476,15 @@ void Solver::enqueue_vcycle(int k, int B, bool guess, cudaStream_t s) {
     return;
   }
   const RowDiv rd(G.nx / 2);
-  const dim3 gs(grid1(G.half()), B);
+  const RowGrid gs(G.half(), B);
   if constexpr (sizeof(T) == sizeof(float)) {
     const LegTile t = make_leg_tile(G, B);
     if (leg_[k] && leg_pays(G, B, t)) {
       // pre-sweeps + restriction (x -> x2), the coarse levels, prolongation +
       // post-sweeps (x2 -> x); k_leg starts after the first red half-sweep
       if (!guess)
-        k_smooth<T><<<gs, kBlock, 0, s>>>(counter_, G, rd, 0, active_, (const T*)L.J, (const T*)L.b,
-                                         (T*)L.x);
+        k_smooth<T><<<gs.grid, gs.threads, 0, s>>>(counter_, G, rd, 0, active_, (const T*)L.J,
+                                                   (const T*)L.b, (T*)L.x);
       const dim3 gl(t.blocks(), B);
       k_leg<false><<<gl, 32 * kLegWarps, kLegSmem, s>>>(counter_, G, C.g, t, active_, (const T*)L.J, (const T*)L.b,
                                         (const T*)L.x, (T*)L.x2, nullptr, (const T*)C.J, (T*)C.b,
@@ -498,17 +498,19 @@ void Solver::enqueue_vcycle(int k, int B, bool guess, cudaStream_t s) {
   }
   auto sweeps = [&](int first, int n) {
     for (int h = first; h < 2 * n; ++h)
-      k_smooth<T><<<gs, kBlock, 0, s>>>(counter_, G, rd, h & 1, active_, (const T*)L.J, (const T*)L.b,
-                                       (T*)L.x);
+      k_smooth<T><<<gs.grid, gs.threads, 0, s>>>(counter_, G, rd, h & 1, active_, (const T*)L.J,
+                                                 (const T*)L.b, (T*)L.x);
   };
   // the guess is zero after its first red half-sweep (x_red = b_red)
   sweeps(guess ? 1 : 0, cfg_.nu1);
-  k_resid_restrict<T><<<dim3(grid1(kRestrictThreads<T> * (int64_t)C.g.ncell()), B), kBlock, 0, s>>>(
+  const RowGrid gr(kRestrictThreads<T> * (int64_t)C.g.ncell(), B);
+  k_resid_restrict<T><<<gr.grid, gr.threads, 0, s>>>(
       counter_, G, C.g, RowDiv(C.g.nx), active_, (const T*)L.J, (const T*)L.b, (const T*)L.x,
       (const T*)C.J, (T*)C.b, (T*)C.x, cfg_.nu1 > 0, cfg_.nu1 > 0);
   enqueue_vcycle<T>(k - 1, B, cfg_.nu1 > 0, s);
   const int black_only = cfg_.nu2 > 0;
-  k_prolong<T><<<dim3(grid1(black_only ? G.half() : G.ncell()), B), kBlock, 0, s>>>(
+  const RowGrid gp(black_only ? G.half() : G.ncell(), B);
+  k_prolong<T><<<gp.grid, gp.threads, 0, s>>>(
       counter_, C.g, G, rd, active_, (const T*)C.x, (T*)L.x, black_only);
   sweeps(0, cfg_.nu2);
 }
@@ -649,8 +651,9 @@ void Solver::enqueue_solve_update(int B, cudaStream_t s) {
   else
     enqueue_vcycles<T>(B, s);
   MGLevel& F = levels_.back();
-  k_update<T><<<dim3(grid1(F.g.half()), B), kBlock, 0, s>>>(counter_, F.g, RowDiv(F.g.nx / 2), active_,
-                                                            (const T*)F.x, F.p, F.c);
+  const RowGrid gu(F.g.half(), B);
+  k_update<T><<<gu.grid, gu.threads, 0, s>>>(counter_, F.g, RowDiv(F.g.nx / 2), active_, (const T*)F.x,
+                                             F.p, F.c);
 }
 
 // Inputs of k_residual on the finest level's workspace.
@@ -1019,7 +1022,8 @@ template <typename T>
 void Solver::launch_timed(int which, int B, cudaStream_t s) {
   MGLevel& F = levels_.back();
   if (which == 0) {
-    k_smooth<T><<<dim3(grid1(F.g.half()), B), kBlock, 0, s>>>(
+    const RowGrid gs(F.g.half(), B);
+    k_smooth<T><<<gs.grid, gs.threads, 0, s>>>(
         counter_, F.g, RowDiv(F.g.nx / 2), 0, active_, (const T*)F.J, (const T*)F.b, (T*)F.x);
   } else if (which == 2) {
     launch_resid<T>(B, s);

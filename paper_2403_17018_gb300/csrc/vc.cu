@@ -487,7 +487,7 @@ void VcSolver::enqueue_linear(int B, cudaStream_t s) {
   double *r = kv_[0], *rh = kv_[1], *pv = kv_[2], *v = kv_[3], *t = kv_[4], *xk = kv_[5];
   const dim3 gd(kry_nchunk_, B);
   const int gs = grid1(B);
-  const dim3 gh(grid1(G_.half()), B);
+  const RowGrid gh(G_.half(), B);
   const RowDiv rd(G_.nx / 2);
   auto upd = [&](int op) {
     k_kry_update<double><<<gv, kBlock, 0, s>>>(counter_, n2, G_.half(), B, op, active_, kS_, r, rh,
@@ -495,7 +495,7 @@ void VcSolver::enqueue_linear(int B, cudaStream_t s) {
   };
   auto precond = [&]() {   // x starts as zero after the first red half-sweep
     for (int h = 1; h < 2 * sweeps_; ++h)
-      k_smooth<double><<<gh, kBlock, 0, s>>>(counter_, G_, rd, h & 1, active_, J_, b_, x_);
+      k_smooth<double><<<gh.grid, gh.threads, 0, s>>>(counter_, G_, rd, h & 1, active_, J_, b_, x_);
   };
   upd(0);
   for (int it = 0; it < kry_; ++it) {
@@ -549,8 +549,9 @@ int VcSolver::run(const double* xi, int B, double* q, double* c_out, double* p_o
       VCK(cudaStreamSynchronize(s));
       if (host_[0] == 0) break;
       enqueue_linear(B, s);
-      k_update<double><<<dim3(grid1(G_.half()), B), kBlock, 0, s>>>(counter_, G_, RowDiv(G_.nx / 2),
-                                                                    active_, x_, p_, c_);
+      const RowGrid gu(G_.half(), B);
+      k_update<double><<<gu.grid, gu.threads, 0, s>>>(counter_, G_, RowDiv(G_.nx / 2), active_, x_, p_,
+                                                      c_);
     }
     k_end_step<<<1, 32, 0, s>>>(counter_, step_);
   }
