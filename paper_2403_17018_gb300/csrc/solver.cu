@@ -84,8 +84,8 @@ Solver::Solver(const henry_config& cfg, int nx, int ny, int nt) : cfg_(cfg), nt_
   tile_r_ = make_res_tile(fine.nx, fine.ny, res_cols_, cfg.res_rows, false);
   tile_j_ = make_res_tile(fine.nx, fine.ny, 2, cfg.res_rows, true);
   nchunk_ = cfg.jac_lag ? tile_r_.tiles() : tile_j_.tiles();
-  // tall default tiles of the residual-only kernel are shared by warps where the batch is small
-  res_split_ = res_cols_ == 4 && cfg.res_rows == 0 && tile_r_.R == 16;
+  // tall tiles of the residual-only kernel are shared by warps where the batch is small
+  res_split_ = res_cols_ == 4 && tile_r_.R >= 16 && tile_r_.R % kResSplit == 0;
   ks_ = 0;
   kc_ = 0;
   for (size_t k = 0; k < geoms_.size(); ++k) {
