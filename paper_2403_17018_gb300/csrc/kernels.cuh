@@ -489,9 +489,10 @@ constexpr int kInvThreadsMost = 256;
 inline int inv_threads(int n, int B) { return n > 24 && B <= 2 * 152 ? kInvThreadsMost : kInvThreads; }
 
 template <typename T>
-__host__ __device__ inline size_t coarse_inv_smem_bytes(int n) {
+__host__ __device__ constexpr size_t coarse_inv_smem_bytes(int n) {
   return ((size_t)n * (n + 1) + n) * sizeof(T) + 2 * (size_t)n * sizeof(int);
 }
+static_assert(coarse_inv_smem_bytes<double>(kMaxCoarseUnknowns) <= 48 * 1024, "no raised limit");
 
 // |v| as an integer of the same order; a NaN comes before everything.
 __device__ __forceinline__ long long magnitude_key(double v) {

@@ -179,13 +179,6 @@ static cudaError_t raise_smem_limit(const void* fn, size_t smem) {
 }
 
 int Solver::ensure(int B, cudaStream_t s) {
-  {
-    const bool f32 = tsize_ == sizeof(float);
-    const int n = 2 * geoms_[0].ncell();
-    const size_t smem = f32 ? coarse_inv_smem_bytes<float>(n) : coarse_inv_smem_bytes<double>(n);
-    CK(raise_smem_limit(f32 ? (const void*)k_coarse_ops<float> : (const void*)k_coarse_ops<double>, smem));
-    CK(raise_smem_limit(f32 ? (const void*)k_coarse_inv<float> : (const void*)k_coarse_inv<double>, smem));
-  }
   if (ks_ > 0) {
     SmallMG<float> Mf;
     SmallMG<double> Md;
