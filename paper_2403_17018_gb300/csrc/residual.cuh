@@ -282,7 +282,10 @@ k_residual(unsigned long long* ctr, Phys P, Geom G, double vtau, ResTile tl, Res
           edgeP = P.Ly - (jw + 0.5) * G.hy;
           if (!J) edgeP = P.drho * P.g * edgeP;
         }
-        const int64_t e = o - col * C + (int64_t)jw * nx;
+        // the tile's first column in row jw, by the form that compiles to the shorter launch
+        // (FP32 Jacobian, 1024x512 x 16, us: 951 so, 993 by the other; FP64, 32x16 x 1024: 200, 189)
+        const int64_t e = TF ? (int64_t)b * ncell + (int64_t)jw * nx + bx * tl.lpr * C
+                             : o - col * C + (int64_t)jw * nx;
         if (bx == 0) {
           w0 = A.qin[(int64_t)b * ny + jw];
           w1 = dcoL * A.phi[e];
