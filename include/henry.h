@@ -162,7 +162,9 @@ typedef struct henry_config {
   int res_rows;         /* rows of cells one thread of the residual/Jacobian
                            kernel walks (its tile height per row group),
                            1..64; 0 (default): 2..16 by the size of the
-                           grid. A schedule knob for the autotuner: it
+                           grid; up to four warps share the rows of heights
+                           of 16 and more that four divides, where the batch
+                           is small. A schedule knob for the autotuner: it
                            trades warps per sample against recomputed faces
                            at tile edges */
   int discretisation;   /* HENRY_DISC_CELL (default) or HENRY_DISC_VERTEX:
