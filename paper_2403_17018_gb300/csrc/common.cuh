@@ -215,7 +215,7 @@ struct ResArgs {
   const double* c_old;    // old time level (otherwise)
   const double* phi;
   const double* K;        // OWN only
-  const double* tx;       // face constants (without OWN), dx and dy halved; the
+  const double* tx;       // face constants (without OWN), dx and dy halves; the
   const double* dx;       //   last column's east slots hold the right side's
   const double* ty;
   const double* dy;

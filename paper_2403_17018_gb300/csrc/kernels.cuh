@@ -115,12 +115,12 @@ static __global__ void k_coarsen_fields(unsigned long long* ctr, Geom Gf, Geom G
   Kc[idx] = 0.25 * (Kf[f0] + Kf[f0 + 1] + Kf[f0 + Gf.nx] + Kf[f0 + Gf.nx + 1]);
 }
 
-// dxh, dyh (optional): the halves of dx, dy; tf (optional): all four in FP32.
+// scale: of dx and dy (the finest level keeps their halves, see ResArgs); tf
+// (optional): all four in FP32, unscaled.
 static __global__ void k_face_consts(unsigned long long* ctr, Phys P, Geom G, int B,
                               const double* __restrict__ phi, const double* __restrict__ K,
                               double* __restrict__ tx, double* __restrict__ dx,
-                              double* __restrict__ ty, double* __restrict__ dy,
-                              double* __restrict__ dxh, double* __restrict__ dyh,
+                              double* __restrict__ ty, double* __restrict__ dy, double scale,
                               float4* __restrict__ tf) {
   HENRY_COUNT_LAUNCH(ctr);
   const int64_t n = (int64_t)B * G.ncell();
@@ -133,13 +133,9 @@ static __global__ void k_face_consts(unsigned long long* ctr, Phys P, Geom G, in
   double a, d, e, f;
   face_constants(P, G, i, j, phi + o, K + o, a, d, e, f);
   tx[idx] = a;
-  dx[idx] = d;
+  dx[idx] = scale * d;
   ty[idx] = e;
-  dy[idx] = f;
-  if (dxh) {
-    dxh[idx] = 0.5 * d;
-    dyh[idx] = 0.5 * f;
-  }
+  dy[idx] = scale * f;
   if (tf) tf[idx] = make_float4((float)a, (float)d, (float)e, (float)f);
 }
 
@@ -1809,8 +1805,7 @@ static __global__ void k_adj_sens(unsigned long long* ctr, Phys P, Geom G, SensC
                            const double* __restrict__ p, const double* __restrict__ c,
                            const double* __restrict__ c_old, const double* __restrict__ phi,
                            const double* __restrict__ K, const double* __restrict__ tx,
-                           const double* __restrict__ dx, const double* __restrict__ ty,
-                           const double* __restrict__ dy, const double* __restrict__ lam,
+                           const double* __restrict__ ty, const double* __restrict__ lam,
                            double* __restrict__ gK, double* __restrict__ gphi,
                            double* __restrict__ gq) {
   HENRY_COUNT_LAUNCH(ctr);

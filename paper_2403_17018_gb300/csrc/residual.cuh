@@ -163,13 +163,13 @@ __device__ __forceinline__ void own_face(double ck, double cd, double k1, double
 constexpr int res_min_blocks(int C, bool J, bool own) { return J ? 8 : (own ? 12 : C == 4 ? 8 : 16); }
 constexpr int kResSplitSlots = 152 * res_min_blocks(4, false, false);   // warps resident
 
-template <typename T, int C, bool J, bool NAT, bool OWN, bool V, bool SPLIT = false>
+template <typename T, int C, bool J, bool NAT, bool OWN, bool V, bool SPLIT = false, bool F32 = true>
 __global__ void __launch_bounds__(SPLIT ? 32 * kResSplit : 32, res_min_blocks(C, J, OWN) / (SPLIT ? kResSplit : 1))
 k_residual(unsigned long long* ctr, Phys P, Geom G, double vtau, ResTile tl, ResArgs A,
            T* __restrict__ Jm, T* __restrict__ bvec, T* __restrict__ xvec) {
   HENRY_COUNT_LAUNCH(ctr);
   constexpr bool PRE = !J && !NAT;                           // mo, so given
-  constexpr bool TF = J && sizeof(T) == 4;                   // face constants in FP32 given
+  constexpr bool TF = J && sizeof(T) == 4 && F32;            // face constants in FP32 given
   const int b = blockIdx.y;
   if (A.active && !A.active[b]) return;
   if (A.refresh && !A.refresh[b]) return;
@@ -591,6 +591,11 @@ k_residual(unsigned long long* ctr, Phys P, Geom G, double vtau, ResTile tl, Res
     for (int s = 16; s > 0; s >>= 1) v += __shfl_down_sync(0xffffffffu, v, s);
     if (lane == 0) A.partial[(int64_t)b * gridDim.x + blockIdx.x] = v;
   }
+}
+
+static __global__ void k_scale(int64_t n, double f, double* __restrict__ v) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) v[i] *= f;
 }
 
 // Face fluxes of the state (p, c), as the residual-only form evaluates them

@@ -162,6 +162,15 @@ int Solver::debug_copy(int mg_level, int what, void* dst, int64_t bytes) const {
     k_face_fluxes<<<grid1((int64_t)n), kBlock>>>(phys_, L.g, cap_, L.p, L.c, L.tx, L.ty, L.qx, L.qy);
     CK(cudaGetLastError());
   }
+  if ((what == 8 || what == 10) && mg_level == (int)levels_.size() - 1) {   // kept as halves
+    double* d = what == 8 ? L.dx : L.dy;
+    k_scale<<<grid1((int64_t)n), kBlock>>>((int64_t)n, 2.0, d);
+    const cudaError_t e = cudaMemcpy(dst, d, nb, cudaMemcpyDefault);
+    k_scale<<<grid1((int64_t)n), kBlock>>>((int64_t)n, 0.5, d);
+    CK(e);
+    CK(cudaDeviceSynchronize());
+    return HENRY_OK;
+  }
   CK(cudaMemcpy(dst, src[what], nb, cudaMemcpyDefault));
   return HENRY_OK;
 }
@@ -246,7 +255,7 @@ int Solver::ensure(int B, cudaStream_t s) {
     lo[k].J = take(kJP * n * tsize_);
     lo[k].b = take(2 * n * tsize_);
     lo[k].x = take(2 * n * tsize_);
-    lo[k].x2 = take(tb_[k] || leg_[k] ? 2 * n * tsize_ : 0);   // second iterate of a leg
+    lo[k].x2 = take(tb_[k] ? 2 * n * tsize_ : 0);   // second iterate of a blocked leg
     lo[k].p = take(n * 8);
     lo[k].c = take(n * 8);
     lo[k].phi = take(n * 8);
@@ -267,9 +276,6 @@ int Solver::ensure(int B, cudaStream_t s) {
   const size_t o_mo = take((size_t)F.ncell() * Bz * 8);
   const size_t o_so = take((size_t)F.ncell() * Bz * 8);
   const size_t o_vt = take((size_t)F.ncell() * Bz * 8);
-  const size_t o_dxh = take((size_t)F.ncell() * Bz * 8);
-  const size_t o_dyh = take((size_t)F.ncell() * Bz * 8);
-  const size_t o_tf = take(tsize_ == sizeof(float) ? (size_t)F.ncell() * Bz * 16 : 0);
   const size_t o_step = take(8);
   const size_t o_qin = take((size_t)F.ny * Bz * 8);
   const size_t o_qin0 = take((size_t)F.ny * Bz * 8);
@@ -297,7 +303,22 @@ int Solver::ensure(int B, cudaStream_t s) {
   const size_t o_ks = take(cfg_.krylov_iters ? Bz * kKryS * 8 : 0);
   const size_t o_kp = take(cfg_.krylov_iters ? 2 * Bz * kry_nchunk_ * 8 : 0);
   const size_t o_ctr = take(8);
-  CK(cudaMalloc(&arena_, off));
+  // what only speeds a solve up comes last, and is left out where the memory ends before it: the
+  // FP32 copies of the face constants (converted in the rebuilds then) and the second iterates of
+  // the legs in one launch (launches per operation then); the values are the same without either
+  const size_t lean = off;
+  const size_t o_tf = take(tsize_ == sizeof(float) ? (size_t)F.ncell() * Bz * 16 : 0);
+  for (size_t k = 0; k < levels_.size(); ++k)
+    if (leg_[k] && !tb_[k]) lo[k].x2 = take(2 * (size_t)levels_[k].g.ncell() * Bz * tsize_);
+  const cudaError_t full = cudaMalloc(&arena_, off);
+  const bool fits = full == cudaSuccess;
+  if (full == cudaErrorMemoryAllocation && lean < off) {
+    cudaGetLastError();
+    off = lean;
+    CK(cudaMalloc(&arena_, off));
+  } else {
+    CK(full);
+  }
   CK(cudaHostAlloc((void**)&n_active_host_, 2 * sizeof(int), cudaHostAllocDefault));
   char* a = (char*)arena_;
   for (size_t k = 0; k < levels_.size(); ++k) {
@@ -315,7 +336,7 @@ int Solver::ensure(int B, cudaStream_t s) {
     L.dy = (double*)(a + lo[k].dy);
     L.qx = (double*)(a + lo[k].qx);
     L.qy = (double*)(a + lo[k].qy);
-    L.x2 = tb_[k] || leg_[k] ? a + lo[k].x2 : nullptr;
+    L.x2 = tb_[k] || (leg_[k] && fits) ? a + lo[k].x2 : nullptr;
   }
   c_old_ = (double*)(a + o_cold);
   p_prev_ = (double*)(a + o_pprev);
@@ -328,9 +349,7 @@ int Solver::ensure(int B, cudaStream_t s) {
   mo_ = (double*)(a + o_mo);
   so_ = (double*)(a + o_so);
   vt_ = (double*)(a + o_vt);
-  dxh_ = (double*)(a + o_dxh);
-  dyh_ = (double*)(a + o_dyh);
-  tf_ = tsize_ == sizeof(float) ? (float4*)(a + o_tf) : nullptr;
+  tf_ = tsize_ == sizeof(float) && fits ? (float4*)(a + o_tf) : nullptr;
   step_ = (int*)(a + o_step);
   qin_ = (double*)(a + o_qin);
   qin0_ = (double*)(a + o_qin0);
@@ -472,7 +491,7 @@ void Solver::enqueue_vcycle(int k, int B, bool guess, cudaStream_t s) {
   const RowGrid gs(G.half(), B);
   if constexpr (sizeof(T) == sizeof(float)) {
     const LegTile t = make_leg_tile(G, B);
-    if (leg_[k] && leg_pays(G, B, t)) {
+    if (leg_[k] && L.x2 && leg_pays(G, B, t)) {
       // pre-sweeps + restriction (x -> x2), the coarse levels, prolongation +
       // post-sweeps (x2 -> x); k_leg starts after the first red half-sweep
       if (!guess)
@@ -659,9 +678,9 @@ ResArgs Solver::res_args() const {
   a.phi = F.phi;
   a.K = F.K;
   a.tx = F.tx;
-  a.dx = dxh_;
+  a.dx = F.dx;
   a.ty = F.ty;
-  a.dy = dyh_;
+  a.dy = F.dy;
   a.tf = tf_;
   a.qin = qin_;
   a.vt = vt_;
@@ -696,7 +715,11 @@ void Solver::launch_resjac(int B, const int* refresh, double* partial, cudaStrea
   ResArgs a = res_args();
   a.refresh = refresh;
   a.partial = partial;
-  k_residual<T, 2, true, false, false, true><<<dim3(tile_j_.tiles(), B), 32, 0, s>>>(
+  // (FP32 without room for the converted face constants: as double and cast)
+  auto kern = k_residual<T, 2, true, false, false, true>;
+  if constexpr (sizeof(T) == sizeof(float))
+    if (!tf_) kern = k_residual<T, 2, true, false, false, true, false, false>;
+  kern<<<dim3(tile_j_.tiles(), B), 32, 0, s>>>(
       counter_, phys_, F.g, F.g.hx * F.g.hy / tau_, tile_j_, a, (T*)F.J, (T*)F.b, (T*)F.x);
 }
 
@@ -914,8 +937,8 @@ int Solver::setup_t(const double* xi, const double* logk, int B, cudaStream_t s)
   for (int k = 0; k < nl; ++k) {
     MGLevel& L = levels_[k];
     k_face_consts<<<grid1((int64_t)B * L.g.ncell()), kBlock, 0, s>>>(
-        counter_, phys_, L.g, B, L.phi, L.K, L.tx, L.dx, L.ty, L.dy, k == nl - 1 ? dxh_ : nullptr,
-        k == nl - 1 ? dyh_ : nullptr, k == nl - 1 ? tf_ : nullptr);
+        counter_, phys_, L.g, B, L.phi, L.K, L.tx, L.dx, L.ty, L.dy, k == nl - 1 ? 0.5 : 1.0,
+        k == nl - 1 ? tf_ : nullptr);
   }
   k_init_state<<<grid1((int64_t)B * G.ncell()), kBlock, 0, s>>>(counter_, phys_, G, B, F.p, F.c,
                                                                 iters_w_, step_);
@@ -1296,7 +1319,7 @@ int Solver::adjoint_t(const double* xi, const double* logk, int B, int qoi, int 
                               2.0 * G.hy * phys_.D / G.hx, 2.0 * G.hy / (phys_.mu * G.hx)};
       k_adj_sens<<<grid1((int64_t)n), kBlock, 0, s>>>(counter_, phys_, G, sens, qfac, B, F.p, F.c,
                                                       c_old_,
-                                                      F.phi, F.K, F.tx, F.dx, F.ty, F.dy, lam_, gK_,
+                                                      F.phi, F.K, F.tx, F.ty, lam_, gK_,
                                                       gphi_, gq_);
       if (st > 1)
         k_adj_prev_rhs<<<grid1((int64_t)n), kBlock, 0, s>>>(counter_, phys_, G, tau_, B, F.phi,

@@ -21,12 +21,12 @@ struct MGLevel {
   void* J = nullptr;     // T [B][20][ncell], colour-split planes
   void* b = nullptr;     // T [B][2][ncell]
   void* x = nullptr;     // T [B][2][ncell]
-  void* x2 = nullptr;    // T [B][2][ncell], the other copy for temporally blocked legs
+  void* x2 = nullptr;    // T [B][2][ncell], the other copy for blocked legs, or null
   double* p = nullptr;   // state at this level (finest: the solver's p)
   double* c = nullptr;
   double* phi = nullptr;
   double* K = nullptr;
-  double* tx = nullptr;  // face constants
+  double* tx = nullptr;  // face constants (finest: the halves of dx and dy)
   double* dx = nullptr;
   double* ty = nullptr;
   double* dy = nullptr;
@@ -169,8 +169,7 @@ class Solver {
   double* mo_ = nullptr;        // old-time storage terms of the step (k_residual)
   double* so_ = nullptr;
   double* vt_ = nullptr;        // V phi / tau per cell (k_residual)
-  double *dxh_ = nullptr, *dyh_ = nullptr;   // halves of the finest dx, dy (k_residual)
-  float4* tf_ = nullptr;        // FP32 face constants of the finest level (FP32 multigrid)
+  float4* tf_ = nullptr;        // FP32 face constants of the finest level (FP32 multigrid), or null
   int* step_ = nullptr;         // completed steps of the current solve (device)
   double* qin_ = nullptr;
   double* qin0_ = nullptr;     // inflow base of the paper field model (time factor per step)
